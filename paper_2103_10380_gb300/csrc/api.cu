@@ -192,8 +192,9 @@ static fnr_status build_from_arrays(fnr_cache *c, const fnr_cache_source *src, c
     float *scales = reinterpret_cast<float *>(base + L.off_scales);
     cudaError_t e;
     const bool dev = src->location == FNR_LOC_DEVICE;
-    // Slab size for staging host arrays (cells per slab).
-    const int64_t slab = dev ? k3 : std::max<int64_t>(1, std::min<int64_t>(k3, (int64_t(256) << 20) / (4 * (nch + 1))));
+    // Slab size for staging host arrays (cells per slab, whole x-rows).
+    const int64_t fit = (int64_t(256) << 20) / (4 * (nch + 1)) / d.k * d.k;
+    const int64_t slab = dev ? k3 : std::max<int64_t>(d.k, std::min<int64_t>(k3, fit));
     DevBuf stage;
     if (!dev) {
         if ((e = dev_malloc(&stage.p, size_t(slab) * 4 * (nch + 1))) != cudaSuccess) return cuda_fail(e, "staging");
@@ -216,15 +217,16 @@ static fnr_status build_from_arrays(fnr_cache *c, const fnr_cache_source *src, c
     const int osh = offset_shift(d.k), odim = (d.k + (1 << osh) - 1) >> osh, ostride = offset_stride(d.D);
     uint16_t *offs = reinterpret_cast<uint16_t *>(base + L.off_offs);
     if (prec == FNR_PREC_FP8_E4M3) {
-        // (1) per offset brick and channel the min and max, then the binary16 midranges; (2) the
-        // per-channel absmax of the density and of the residuals; (3) the scales
+        // (1) per offset brick and channel the min and max, and the absmax of the density; (2) the binary16
+        // midranges and, from the same extremes, the absmax of the residuals; (3) the scales
         const int64_t nbo3 = int64_t(odim) * odim * odim;
         DevBuf amax, kmm;
         if ((e = dev_malloc(&amax.p, sizeof(unsigned) * (1 + nch))) != cudaSuccess) return cuda_fail(e, "absmax");
         if ((e = dev_malloc(&kmm.p, sizeof(unsigned) * 2 * size_t(nbo3) * nch)) != cudaSuccess)
             return cuda_fail(e, "offset min / max");
         unsigned *kmin = static_cast<unsigned *>(kmm.p), *kmax = kmin + size_t(nbo3) * nch;
-        if ((e = cudaMemsetAsync(amax.p, 0, sizeof(unsigned) * (1 + nch), s)) != cudaSuccess ||
+        unsigned *amx = static_cast<unsigned *>(amax.p);
+        if ((e = cudaMemsetAsync(amx, 0, sizeof(unsigned) * (1 + nch), s)) != cudaSuccess ||
             (e = cudaMemsetAsync(kmin, 0xff, sizeof(unsigned) * size_t(nbo3) * nch, s)) != cudaSuccess ||
             (e = cudaMemsetAsync(kmax, 0, sizeof(unsigned) * size_t(nbo3) * nch, s)) != cudaSuccess)
             return cuda_fail(e, "memset");
@@ -232,33 +234,15 @@ static fnr_status build_from_arrays(fnr_cache *c, const fnr_cache_source *src, c
             const int64_t n = std::min(slab, k3 - c0);
             const float *sp, *up;
             if ((e = slab_ptrs(c0, n, &sp, &up)) != cudaSuccess) return cuda_fail(e, "upload");
-            if ((e = launch_brick_minmax(up, c0, n, d.k, nch, osh, odim, kmin, kmax, s)) != cudaSuccess)
+            if ((e = launch_brick_minmax(up, c0 / d.k, (c0 + n) / d.k, d.k, nch, osh, odim, kmin, kmax, s)) !=
+                    cudaSuccess ||
+                (e = launch_sigma_absmax(sp, n, amx, s)) != cudaSuccess)
                 return cuda_fail(e, "offset min / max kernel");
             if (!dev && (e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "min / max sync");
         }
-        if ((e = launch_brick_offsets(kmin, kmax, nbo3, nch, offs, ostride, s)) != cudaSuccess)
+        if ((e = launch_brick_offsets(kmin, kmax, nbo3, nch, offs, ostride, amx, s)) != cudaSuccess)
             return cuda_fail(e, "offsets kernel");
-        for (int64_t c0 = 0; c0 < k3; c0 += slab) {
-            const int64_t n = std::min(slab, k3 - c0);
-            const float *sp, *up;
-            if ((e = slab_ptrs(c0, n, &sp, &up)) != cudaSuccess) return cuda_fail(e, "upload");
-            // the density channel (and the raw absmax of the others, overwritten below)
-            if ((e = launch_absmax(sp, up, n, nch, static_cast<unsigned *>(amax.p), s)) != cudaSuccess)
-                return cuda_fail(e, "absmax kernel");
-            if (!dev && (e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "absmax sync");
-        }
-        if ((e = cudaMemsetAsync(static_cast<unsigned *>(amax.p) + 1, 0, sizeof(unsigned) * nch, s)) != cudaSuccess)
-            return cuda_fail(e, "memset");
-        for (int64_t c0 = 0; c0 < k3; c0 += slab) {
-            const int64_t n = std::min(slab, k3 - c0);
-            const float *sp, *up;
-            if ((e = slab_ptrs(c0, n, &sp, &up)) != cudaSuccess) return cuda_fail(e, "upload");
-            if ((e = launch_residual_absmax(up, c0, n, d.k, nch, offs, osh, odim, ostride,
-                                            static_cast<unsigned *>(amax.p), s)) != cudaSuccess)
-                return cuda_fail(e, "residual absmax kernel");
-            if (!dev && (e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "residual sync");
-        }
-        if ((e = launch_scales_from_absmax(static_cast<unsigned *>(amax.p), scales, 1 + nch, s)) != cudaSuccess)
+        if ((e = launch_scales_from_absmax(amx, scales, 1 + nch, s)) != cudaSuccess)
             return cuda_fail(e, "scales kernel");
         if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "scales sync");
     }
@@ -269,8 +253,8 @@ static fnr_status build_from_arrays(fnr_cache *c, const fnr_cache_source *src, c
         if ((e = launch_convert_sigma(sp, base + L.off_sigma + c0 * elem_bytes(prec), n, prec, scales, s)) !=
             cudaSuccess)
             return cuda_fail(e, "density conversion");
-        if ((e = launch_convert_uvw(up, base + L.off_uvw + c0 * L.rec_stride, n, d.D, prec, L.rec_stride, scales,
-                                    s, offs, c0, d.k, osh, odim, ostride)) != cudaSuccess)
+        if ((e = launch_convert_uvw(up, base + L.off_uvw + c0 * L.rec_stride, c0 / d.k, (c0 + n) / d.k, d.k, d.D, prec,
+                                    L.rec_stride, scales, offs, osh, odim, ostride, s)) != cudaSuccess)
             return cuda_fail(e, "uvw conversion");
         if (!dev && (e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "conversion sync");
     }

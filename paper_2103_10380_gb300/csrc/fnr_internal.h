@@ -125,23 +125,22 @@ cudaError_t launch_gather_bricks(const void *sigma, const char *uvw, void *sigma
                                  int s_sigma, int rec_stride, cudaStream_t s);
 cudaError_t launch_convert_sigma(const float *in, void *out, int64_t n, int prec, const float *scale,
                                  cudaStream_t s);
-cudaError_t launch_convert_uvw(const float *in, char *out, int64_t n_cells, int D, int prec, int rec_stride,
-                               const float *scales, cudaStream_t s, const uint16_t *offs = nullptr,
-                               int64_t c0 = 0, int k = 0, int oshift = 0, int odim = 0, int ostride = 0);
+// The records of the x-rows [r0, r1) (row z k + y; `in` and `out` point at row r0).
+cudaError_t launch_convert_uvw(const float *in, char *out, int64_t r0, int64_t r1, int k, int D, int prec,
+                               int rec_stride, const float *scales, const uint16_t *offs, int oshift, int odim,
+                               int ostride, cudaStream_t s);
 // E4M3 (u, v, w) offsets: the smallest power of two >= 4 with ceil(k / Bo) <= 64, as a shift.
 int offset_shift(int k);
-// Per offset brick and channel: running min / max of a slab of cells c0 .. c0 + n (order-preserving
-// uint keys; initialise with 0xffffffff / 0), then the binary16 midranges.
-cudaError_t launch_brick_minmax(const float *uvw, int64_t c0, int64_t n, int k, int nch, int oshift, int odim,
+// Per offset brick and channel: running min / max of the x-rows [r0, r1) (`uvw` points at row r0;
+// order-preserving uint keys, initialise with 0xffffffff / 0), then the binary16 midranges and each
+// channel's absmax of the residuals from them (atomicMax on the bits of |r|, amax_bits[1 + c]).
+cudaError_t launch_brick_minmax(const float *uvw, int64_t r0, int64_t r1, int k, int nch, int oshift, int odim,
                                 unsigned *kmin, unsigned *kmax, cudaStream_t s);
 cudaError_t launch_brick_offsets(const unsigned *kmin, const unsigned *kmax, int64_t n_bricks, int nch,
-                                 uint16_t *offs, int ostride, cudaStream_t s);
-// Per-channel absmax of the residuals from the offsets (atomicMax on the bits of |r|, amax_bits[1 + c]).
-cudaError_t launch_residual_absmax(const float *uvw, int64_t c0, int64_t n, int k, int nch, const uint16_t *offs,
-                                   int oshift, int odim, int ostride, unsigned *amax_bits, cudaStream_t s);
+                                 uint16_t *offs, int ostride, unsigned *amax_bits, cudaStream_t s);
 cudaError_t launch_convert_beta(const float *in, void *out, int64_t n, int prec, cudaStream_t s);
-cudaError_t launch_absmax(const float *sigma, const float *uvw, int64_t n_cells, int nch, unsigned *amax_bits,
-                          cudaStream_t s);
+// Absmax of the clamped densities (atomicMax on the bits, amax_bits[0]).
+cudaError_t launch_sigma_absmax(const float *sigma, int64_t n, unsigned *amax_bits, cudaStream_t s);
 // Brick occupancy bits from a stored density plane (words must be zeroed first).
 cudaError_t launch_occupancy(const CacheView &v, uint32_t *words, cudaStream_t s);
 int occupancy_shift(const fnr_cache_desc *d);

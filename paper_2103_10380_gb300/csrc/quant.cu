@@ -10,8 +10,19 @@
 // The brick occupancy bits are derived from the stored densities with the
 // march's own dequantisation, so "brick empty" means exactly that every
 // density the march could load there is 0.
+//
+// All of this is bound by memory bandwidth (4 (1 + 3D) bytes read per cell and
+// pass), so the kernels over the channels share one mapping: a thread owns a
+// fixed group of VEC consecutive floats of an x-row -- a fixed x, fixed channels
+// and so one brick, one set of offsets and scales -- and walks the rows (y, z) of
+// a square of rows, 64 for the offset bricks of k = 512. Index arithmetic, offset
+// and scale loads are paid once per thread instead of once per element, a warp
+// reads 512 consecutive bytes per row, and the loads of several rows are in
+// flight together. E4M3 reads the source twice (min / max, then codes).
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
+
+#include <algorithm>
 
 #include "fnr_internal.h"
 #include "march_device.cuh"
@@ -41,108 +52,237 @@ __device__ __forceinline__ float from_order_key(unsigned o) {
     return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
 }
 
-// Offset brick of cell index `cell` (x fastest): (z >> sh, y >> sh, x >> sh).
-__device__ __forceinline__ int64_t offset_brick_of(int64_t cell, int k, int sh, int dim) {
-    const int64_t x = cell % k, y = (cell / k) % k, z = cell / (static_cast<int64_t>(k) * k);
-    return ((z >> sh) * dim + (y >> sh)) * dim + (x >> sh);
+// VEC consecutive floats of the source, one load.
+template <int VEC>
+__device__ __forceinline__ void load_floats(const float *__restrict__ p, float (&v)[VEC]) {
+    if constexpr (VEC == 4) {
+        const float4 q = __ldcs(reinterpret_cast<const float4 *>(p));
+        v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
+    } else if constexpr (VEC == 2) {
+        const float2 q = __ldcs(reinterpret_cast<const float2 *>(p));
+        v[0] = q.x, v[1] = q.y;
+    } else {
+        v[0] = __ldcs(p);
+    }
 }
 
-// One thread per cell of the slab, all channels; lanes of a warp whose cells
-// share an offset brick combine their keys first, so each (warp, brick,
-// channel) makes one atomic min and one atomic max.
-__global__ void brick_minmax_kernel(const float *__restrict__ uvw, int64_t c0, int64_t n, int k, int nch, int sh,
-                                    int dim, unsigned *__restrict__ kmin, unsigned *__restrict__ kmax) {
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    const int64_t n_iter = (n + stride - 1) / stride;  // the same trip count for every lane (warp-wide sync)
-    const int64_t first = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    for (int64_t it = 0; it < n_iter; ++it) {
-        const int64_t i = first + it * stride;
-        const bool in = i < n;
-        const long long b = in ? offset_brick_of(c0 + i, k, sh, dim) : -1;
-        const unsigned same = __match_any_sync(0xffffffffu, b);
-        const bool leader = in && (threadIdx.x & 31) == __ffs(same) - 1;
-        for (int c = 0; c < nch; ++c) {
-            const float v = in ? uvw[i * nch + c] : 0.0f;
-            const bool ok = in && v == v;
-            const unsigned lo = __reduce_min_sync(same, ok ? order_key(v) : 0xffffffffu);
-            const unsigned hi = __reduce_max_sync(same, ok ? order_key(v) : 0u);
-            if (leader) {
-                if (lo != 0xffffffffu) atomicMin(kmin + b * nch + c, lo);
-                if (hi != 0u) atomicMax(kmax + b * nch + c, hi);
+// The rows [ya, yb) of plane z that lie in the square of rows (by, .) of side
+// 2^sh and in the slab's rows [r0, r1).
+__device__ __forceinline__ void square_rows(int z, int by, int sh, int k, int64_t r0, int64_t r1, int &ya, int &yb) {
+    const int64_t first = static_cast<int64_t>(z) * k;
+    ya = static_cast<int>(max(static_cast<int64_t>(by << sh), r0 - first));
+    yb = static_cast<int>(min(static_cast<int64_t>(min((by + 1) << sh, k)), r1 - first));
+}
+
+constexpr int kRowThreads = 256;
+
+// Min and max per offset brick and channel (NaN ignored). Block (x, y, z):
+// kRowThreads groups of VEC floats of the rows of offset-brick row (y, bz0 + z);
+// each thread keeps its VEC minima and maxima in registers over the rows (min /
+// max order -0 below +0, as the keys do), the block combines the cells of a brick
+// in shared memory, and one atomic per (block, brick, channel) joins blocks and
+// slabs. A group never crosses a brick: a brick's part of a row is 2^sh nch floats,
+// a multiple of 4. k = 256, D = 8 (1.6 GB) took 2.41 ms with one thread per cell and
+// its channels in a loop; k = 512 (12.9 GB) takes 1.73 ms here (7.4 TB/s read).
+template <int VEC>
+__global__ void __launch_bounds__(kRowThreads)
+    brick_minmax_kernel(const float *__restrict__ uvw, int64_t r0, int64_t r1, int bz0, int k, int nch, int sh,
+                        int dim, unsigned *__restrict__ kmin, unsigned *__restrict__ kmax) {
+    // entries of a block: (bricks it touches) x nch <= VEC kRowThreads / 4 + 2 nch
+    constexpr int kEntries = VEC * kRowThreads / 4 + 2 * 3 * FNR_MAX_D;
+    __shared__ unsigned lo[kEntries], hi[kEntries];
+    const int n_groups = k * nch / VEC;
+    const int g0 = blockIdx.x * kRowThreads, g = g0 + threadIdx.x;
+    const int g_last = min(g0 + kRowThreads, n_groups) - 1;
+    const int b0 = (g0 * VEC / nch) >> sh, n_entries = (((g_last * VEC / nch) >> sh) - b0 + 1) * nch;
+    for (int e = threadIdx.x; e < n_entries; e += kRowThreads) {
+        lo[e] = 0xffffffffu;
+        hi[e] = 0u;
+    }
+    __syncthreads();
+    const int by = blockIdx.y, bz = bz0 + blockIdx.z;
+    if (g < n_groups) {
+        float mn[VEC], mx[VEC];
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) {
+            mn[i] = __int_as_float(0x7f800000);
+            mx[i] = -mn[i];
+        }
+        const int64_t row = static_cast<int64_t>(k) * nch;
+        for (int z = bz << sh; z < min((bz + 1) << sh, k); ++z) {
+            int ya, yb;
+            square_rows(z, by, sh, k, r0, r1, ya, yb);
+            const float *p = uvw + (static_cast<int64_t>(z) * k + ya - r0) * row + g * VEC;
+#pragma unroll 8
+            for (int y = ya; y < yb; ++y, p += row) {
+                float v[VEC];
+                load_floats<VEC>(p, v);
+#pragma unroll
+                for (int i = 0; i < VEC; ++i) {
+                    mn[i] = fminf(mn[i], v[i]);
+                    mx[i] = fmaxf(mx[i], v[i]);
+                }
+            }
+        }
+        const int cell = g * VEC / nch, eb = ((cell >> sh) - b0) * nch;
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) {
+            const int e = eb + (g * VEC + i) % nch;
+            if (mn[i] <= mx[i]) {  // some value was not NaN
+                atomicMin(&lo[e], order_key(mn[i]));
+                atomicMax(&hi[e], order_key(mx[i]));
             }
         }
     }
+    __syncthreads();
+    const int64_t out = ((static_cast<int64_t>(bz) * dim + by) * dim + b0) * nch;
+    for (int e = threadIdx.x; e < n_entries; e += kRowThreads)
+        if (lo[e] != 0xffffffffu) {
+            atomicMin(kmin + out + e, lo[e]);
+            atomicMax(kmax + out + e, hi[e]);
+        }
 }
 
 // Offsets: the binary16 (nearest even) value of (min + max) * 0.5 in binary32, 0 for a brick
-// whose values were all NaN; the padding of each offset record is 0.
+// whose values were all NaN; the padding of each offset record is 0. Each channel's absmax of the
+// residuals |binary32(u - offset)| (NaN skipped) goes to amax_bits[1 + c]: u - offset rounded is
+// monotone in u, so over a brick it is reached at the brick's min or max (an infinite offset makes
+// every residual infinite or NaN, the finite one of the two extremes among them), and no pass
+// over the source is needed. A thread keeps one channel.
 __global__ void brick_offsets_kernel(const unsigned *__restrict__ kmin, const unsigned *__restrict__ kmax,
-                                     int64_t n_bricks, int nch, uint16_t *__restrict__ offs, int ostride) {
-    const int64_t total = n_bricks * ostride;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = e / ostride;
-        const int c = static_cast<int>(e - b * ostride);
-        float m = 0.0f;
-        if (c < nch && kmin[b * nch + c] != 0xffffffffu)
-            m = (from_order_key(kmin[b * nch + c]) + from_order_key(kmax[b * nch + c])) * 0.5f;
-        offs[e] = __half_as_ushort(__float2half_rn(m));
-    }
-}
-
-__device__ __forceinline__ float offset_of(const uint16_t *__restrict__ offs, int64_t cell, int c, int k, int sh,
-                                           int dim, int ostride) {
-    return __half2float(__ushort_as_half(offs[offset_brick_of(cell, k, sh, dim) * ostride + c]));
-}
-
-// Per-channel absmax of |binary32(u - offset)| (NaN skipped) into amax_bits[1 + c].
-__global__ void residual_absmax_kernel(const float *__restrict__ uvw, int64_t c0, int64_t n, int k, int nch,
-                                       const uint16_t *__restrict__ offs, int sh, int dim, int ostride,
-                                       unsigned *__restrict__ amax_bits) {
+                                     int64_t n_bricks, int nch, uint16_t *__restrict__ offs, int ostride,
+                                     unsigned *__restrict__ amax_bits) {
     __shared__ unsigned smax[3 * FNR_MAX_D];
     for (int c = threadIdx.x; c < nch; c += blockDim.x) smax[c] = 0u;
     __syncthreads();
-    const int64_t total = n * nch;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = e / nch;
-        const int c = static_cast<int>(e - i * nch);
-        const float r = fabsf(uvw[e] - offset_of(offs, c0 + i, c, k, sh, dim, ostride));
-        if (r == r) atomicMax(&smax[c], __float_as_uint(r));
+    const int per = blockDim.x / ostride;  // bricks per block and step
+    const int c = threadIdx.x % ostride, lb = threadIdx.x / ostride;
+    if (lb < per) {
+        unsigned big = 0u;
+        for (int64_t b = static_cast<int64_t>(blockIdx.x) * per + lb; b < n_bricks;
+             b += static_cast<int64_t>(gridDim.x) * per) {
+            float m = 0.0f;
+            const unsigned ko = c < nch ? kmin[b * nch + c] : 0xffffffffu;
+            const bool any = ko != 0xffffffffu;
+            float lo = 0.0f, hi = 0.0f;
+            if (any) {
+                lo = from_order_key(ko);
+                hi = from_order_key(kmax[b * nch + c]);
+                m = (lo + hi) * 0.5f;
+            }
+            const __half mh = __float2half_rn(m);
+            offs[b * ostride + c] = __half_as_ushort(mh);
+            if (any) {
+                const float mf = __half2float(mh), rl = fabsf(lo - mf), rh = fabsf(hi - mf);
+                if (rl == rl) big = max(big, __float_as_uint(rl));
+                if (rh == rh) big = max(big, __float_as_uint(rh));
+            }
+        }
+        if (big) atomicMax(&smax[c], big);
     }
     __syncthreads();
-    for (int c = threadIdx.x; c < nch; c += blockDim.x) atomicMax(&amax_bits[1 + c], smax[c]);
+    for (int i = threadIdx.x; i < nch; i += blockDim.x)
+        if (smax[i]) atomicMax(&amax_bits[1 + i], smax[i]);
 }
 
-__global__ void convert_sigma_kernel(const float *__restrict__ in, void *__restrict__ out, int64_t n, int prec,
+// four densities per thread and step when both sides are aligned for it, else one
+template <int PREC, int VEC>
+__global__ void convert_sigma_kernel(const float *__restrict__ in, void *__restrict__ out, int64_t n,
                                      const float *__restrict__ scale) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float v = clamp_density(in[i]);
-        if (prec == FNR_PREC_FP32) static_cast<float *>(out)[i] = v;
-        else if (prec == FNR_PREC_FP16) static_cast<__half *>(out)[i] = __float2half_rn(v);
-        else static_cast<unsigned char *>(out)[i] = to_e4m3(__fdiv_rn(v, scale[0]));
+    const float sc = PREC == FNR_PREC_FP8_E4M3 ? scale[0] : 1.0f;
+    const int64_t groups = n / VEC, stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    const int64_t first = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    auto store = [&](int64_t i, const auto &v) {
+        constexpr int W = sizeof(v) / 4;
+        if constexpr (PREC == FNR_PREC_FP32) {
+            if constexpr (W == 4) reinterpret_cast<float4 *>(out)[i] = make_float4(v[0], v[1], v[2], v[3]);
+            else static_cast<float *>(out)[i] = v[0];
+        } else if constexpr (PREC == FNR_PREC_FP16) {
+            if constexpr (W == 4) {
+                const __half2 a = __floats2half2_rn(v[0], v[1]), b = __floats2half2_rn(v[2], v[3]);
+                reinterpret_cast<uint2 *>(out)[i] =
+                    make_uint2(*reinterpret_cast<const unsigned *>(&a), *reinterpret_cast<const unsigned *>(&b));
+            } else static_cast<__half *>(out)[i] = __float2half_rn(v[0]);
+        } else {
+            unsigned q = 0u;
+#pragma unroll
+            for (int j = 0; j < W; ++j) q |= static_cast<unsigned>(to_e4m3(__fdiv_rn(v[j], sc))) << (8 * j);
+            if constexpr (W == 4) static_cast<unsigned *>(out)[i] = q;
+            else static_cast<unsigned char *>(out)[i] = static_cast<unsigned char>(q);
+        }
+    };
+#pragma unroll 4
+    for (int64_t i = first; i < groups; i += stride) {
+        float v[VEC];
+        load_floats<VEC>(in + i * VEC, v);
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) v[j] = clamp_density(v[j]);
+        store(i, v);
+    }
+    if (VEC > 1 && first < n - groups * VEC) {
+        float v[1] = {clamp_density(in[groups * VEC + first])};
+        store(groups * VEC + first, v);
     }
 }
 
-// One thread per output byte-group would waste bandwidth on the padding; one
-// thread per (cell, channel) element, padding written by channel-0 threads.
-__global__ void convert_uvw_kernel(const float *__restrict__ in, char *__restrict__ out, int64_t n_cells, int nch,
-                                   int prec, int rec_stride, const float *__restrict__ scales,
-                                   const uint16_t *__restrict__ offs, int64_t c0, int k, int sh, int dim,
-                                   int ostride) {
-    const int64_t total = n_cells * nch;
-    const int es = prec == FNR_PREC_FP32 ? 4 : prec == FNR_PREC_FP16 ? 2 : 1;
-    const int pad_bytes = rec_stride - nch * es;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t cell = e / nch;
-        const int ch = static_cast<int>(e - cell * nch);
-        char *rec = out + cell * rec_stride;
-        const float v = in[e];
-        if (prec == FNR_PREC_FP32) reinterpret_cast<float *>(rec)[ch] = v;
-        else if (prec == FNR_PREC_FP16) reinterpret_cast<__half *>(rec)[ch] = __float2half_rn(v);
-        else
-            reinterpret_cast<unsigned char *>(rec)[ch] =
-                to_e4m3(__fdiv_rn(__fsub_rn(v, offset_of(offs, c0 + cell, ch, k, sh, dim, ostride)), scales[1 + ch]));
-        if (ch == 0)
-            for (int b = 0; b < pad_bytes; ++b) rec[nch * es + b] = 0;
+// The records of the rows [r0, r1). VEC divides nch, so a thread's floats are
+// channels c0 .. c0 + VEC - 1 of the cells at one x; the thread of a record's last
+// channels also writes its padding (a multiple of the store's width: both divide
+// the record's alignment). k = 256, D = 8 to E4M3 took 2.44 ms with one thread per
+// element that found its cell, brick, offset and scale anew; k = 512 (16.1 GB read
+// and written) takes 2.94 ms here, to FP16 2.92 ms (19.3 GB), to FP32 3.77 ms (25.8 GB).
+template <int PREC, int VEC>
+__global__ void __launch_bounds__(kRowThreads)
+    convert_uvw_kernel(const float *__restrict__ in, char *__restrict__ out, int64_t r0, int64_t r1, int bz0, int k,
+                       int nch, int rec_stride, const float *__restrict__ scales, const uint16_t *__restrict__ offs,
+                       int sh, int dim, int ostride) {
+    constexpr int kElem = PREC == FNR_PREC_FP32 ? 4 : PREC == FNR_PREC_FP16 ? 2 : 1;
+    constexpr int kBytes = VEC * kElem;
+    const int g = blockIdx.x * kRowThreads + threadIdx.x;
+    if (g >= k * nch / VEC) return;
+    const int by = blockIdx.y, bz = bz0 + blockIdx.z;
+    const int x = g * VEC / nch, c0 = g * VEC - x * nch;
+    const int pad = c0 + VEC == nch ? rec_stride - nch * kElem : 0;
+    float m[VEC], s[VEC];
+    if constexpr (PREC == FNR_PREC_FP8_E4M3) {
+        const int64_t brick = (static_cast<int64_t>(bz) * dim + by) * dim + (x >> sh);
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) {
+            m[i] = __half2float(__ushort_as_half(offs[brick * ostride + c0 + i]));
+            s[i] = scales[1 + c0 + i];
+        }
+    }
+    const int64_t row = static_cast<int64_t>(k) * nch, row_out = static_cast<int64_t>(k) * rec_stride;
+    for (int z = bz << sh; z < min((bz + 1) << sh, k); ++z) {
+        int ya, yb;
+        square_rows(z, by, sh, k, r0, r1, ya, yb);
+        const int64_t r = static_cast<int64_t>(z) * k + ya - r0;
+        const float *p = in + r * row + g * VEC;
+        char *q = out + r * row_out + static_cast<int64_t>(x) * rec_stride + c0 * kElem;
+#pragma unroll 4
+        for (int y = ya; y < yb; ++y, p += row, q += row_out) {
+            float v[VEC];
+            load_floats<VEC>(p, v);
+            auto put = [](char *at, const unsigned (&w)[4]) {
+                if constexpr (kBytes == 16) *reinterpret_cast<uint4 *>(at) = make_uint4(w[0], w[1], w[2], w[3]);
+                else if constexpr (kBytes == 8) *reinterpret_cast<uint2 *>(at) = make_uint2(w[0], w[1]);
+                else if constexpr (kBytes == 4) *reinterpret_cast<unsigned *>(at) = w[0];
+                else if constexpr (kBytes == 2) *reinterpret_cast<uint16_t *>(at) = static_cast<uint16_t>(w[0]);
+                else *reinterpret_cast<unsigned char *>(at) = static_cast<unsigned char>(w[0]);
+            };
+            unsigned w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+            for (int i = 0; i < VEC; ++i) {
+                if constexpr (PREC == FNR_PREC_FP32) w[i] = __float_as_uint(v[i]);
+                else if constexpr (PREC == FNR_PREC_FP16)
+                    w[i >> 1] |= static_cast<unsigned>(__half_as_ushort(__float2half_rn(v[i]))) << (16 * (i & 1));
+                else
+                    w[0] |= static_cast<unsigned>(to_e4m3(__fdiv_rn(__fsub_rn(v[i], m[i]), s[i]))) << (8 * i);
+            }
+            put(q, w);
+            const unsigned zero[4] = {0u, 0u, 0u, 0u};
+            for (int b = 0; b < pad; b += kBytes) put(q + kBytes + b, zero);
+        }
     }
 }
 
@@ -153,27 +293,29 @@ __global__ void convert_beta_kernel(const float *__restrict__ in, void *__restri
     }
 }
 
-// Channel absmax: channel 0 = clamped density, 1..nch = (u, v, w) channels.
-// Non-negative binary32 values order like their bit patterns, so an unsigned
-// atomicMax on the bits is an exact max. NaNs are skipped.
-__global__ void absmax_kernel(const float *__restrict__ sigma, const float *__restrict__ uvw, int64_t n_cells, int nch,
-                              unsigned *__restrict__ amax_bits) {
-    __shared__ unsigned smax[1 + 3 * FNR_MAX_D];
-    for (int c = threadIdx.x; c <= nch; c += blockDim.x) smax[c] = 0u;
+// Absmax of the clamped densities into amax_bits[0]. Non-negative binary32
+// values order like their bit patterns, so an unsigned max of the bits is exact
+// (NaN is clamped to 0).
+template <int VEC>
+__global__ void sigma_absmax_kernel(const float *__restrict__ sigma, int64_t n, unsigned *__restrict__ amax_bits) {
+    __shared__ unsigned smax;
+    if (threadIdx.x == 0) smax = 0u;
     __syncthreads();
-    unsigned local_s = 0u;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_cells; i += (int64_t)gridDim.x * blockDim.x) {
-        const float v = fabsf(clamp_density(sigma[i]));
-        local_s = max(local_s, __float_as_uint(v));
+    unsigned big = 0u;
+    const int64_t groups = n / VEC, stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    const int64_t first = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+#pragma unroll 4
+    for (int64_t i = first; i < groups; i += stride) {
+        float v[VEC];
+        load_floats<VEC>(sigma + i * VEC, v);
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) big = max(big, __float_as_uint(clamp_density(v[j])));
     }
-    atomicMax(&smax[0], local_s);
-    const int64_t total = n_cells * nch;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const float v = fabsf(uvw[e]);
-        if (v == v) atomicMax(&smax[1 + static_cast<int>(e % nch)], __float_as_uint(v));
-    }
+    if (first < n - groups * VEC) big = max(big, __float_as_uint(clamp_density(sigma[groups * VEC + first])));
+    big = __reduce_max_sync(0xffffffffu, big);
+    if ((threadIdx.x & 31) == 0 && big) atomicMax(&smax, big);
     __syncthreads();
-    for (int c = threadIdx.x; c <= nch; c += blockDim.x) atomicMax(&amax_bits[c], smax[c]);
+    if (threadIdx.x == 0 && smax) atomicMax(&amax_bits[0], smax);
 }
 
 __global__ void scales_kernel(const unsigned *__restrict__ amax_bits, float *__restrict__ scales, int n) {
@@ -308,41 +450,99 @@ cudaError_t launch_brick_distance(const uint32_t *words, int nb, int occ_shift, 
     return cudaGetLastError();
 }
 
+namespace {
+
+bool aligned(const void *p, size_t bytes) { return reinterpret_cast<uintptr_t>(p) % bytes == 0; }
+
+// Floats per load for a source at p whose groups must divide `unit` floats.
+int group_width(const float *p, int64_t unit) {
+    if (unit % 4 == 0 && aligned(p, 16)) return 4;
+    return unit % 2 == 0 && aligned(p, 8) ? 2 : 1;
+}
+
+// Blocks over the rows [r0, r1): groups of an x-row, squares of rows along y, the squares along z that the
+// rows reach (the first of them in *bz0).
+dim3 row_grid(int64_t r0, int64_t r1, int k, int nch, int vec, int sh, int *bz0) {
+    *bz0 = static_cast<int>(r0 / k) >> sh;
+    const int bz1 = static_cast<int>((r1 - 1) / k) >> sh;
+    const int groups = k * nch / vec;
+    return dim3(static_cast<unsigned>((groups + kRowThreads - 1) / kRowThreads),
+                static_cast<unsigned>((k + (1 << sh) - 1) >> sh), static_cast<unsigned>(bz1 - *bz0 + 1));
+}
+
+template <int PREC>
+void convert_sigma_p(const float *in, void *out, int64_t n, const float *scale, cudaStream_t s) {
+    constexpr size_t es = PREC == FNR_PREC_FP32 ? 4 : PREC == FNR_PREC_FP16 ? 2 : 1;
+    if (aligned(in, 16) && aligned(out, 4 * es))
+        convert_sigma_kernel<PREC, 4><<<grid_for((n + 3) / 4, 256), 256, 0, s>>>(in, out, n, scale);
+    else
+        convert_sigma_kernel<PREC, 1><<<grid_for(n, 256), 256, 0, s>>>(in, out, n, scale);
+}
+
+template <int PREC>
+void convert_uvw_p(const float *in, char *out, int64_t r0, int64_t r1, int k, int nch, int rec_stride,
+                   const float *scales, const uint16_t *offs, int sh, int dim, int ostride, cudaStream_t s) {
+    const int vec = group_width(in, nch);
+    int bz0;
+    const dim3 grid = row_grid(r0, r1, k, nch, vec, sh, &bz0);
+    if (vec == 4)
+        convert_uvw_kernel<PREC, 4><<<grid, kRowThreads, 0, s>>>(in, out, r0, r1, bz0, k, nch, rec_stride, scales, offs,
+                                                                 sh, dim, ostride);
+    else if (vec == 2)
+        convert_uvw_kernel<PREC, 2><<<grid, kRowThreads, 0, s>>>(in, out, r0, r1, bz0, k, nch, rec_stride, scales, offs,
+                                                                 sh, dim, ostride);
+    else
+        convert_uvw_kernel<PREC, 1><<<grid, kRowThreads, 0, s>>>(in, out, r0, r1, bz0, k, nch, rec_stride, scales, offs,
+                                                                 sh, dim, ostride);
+}
+
+}  // namespace
+
 cudaError_t launch_convert_sigma(const float *in, void *out, int64_t n, int prec, const float *scale, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    convert_sigma_kernel<<<grid_for(n, 256), 256, 0, s>>>(in, out, n, prec, scale);
+    if (prec == FNR_PREC_FP32) convert_sigma_p<FNR_PREC_FP32>(in, out, n, scale, s);
+    else if (prec == FNR_PREC_FP16) convert_sigma_p<FNR_PREC_FP16>(in, out, n, scale, s);
+    else convert_sigma_p<FNR_PREC_FP8_E4M3>(in, out, n, scale, s);
     return cudaGetLastError();
 }
 
-cudaError_t launch_convert_uvw(const float *in, char *out, int64_t n_cells, int D, int prec, int rec_stride,
-                               const float *scales, cudaStream_t s, const uint16_t *offs, int64_t c0, int k,
-                               int oshift, int odim, int ostride) {
-    if (n_cells <= 0) return cudaSuccess;
-    if (prec == FNR_PREC_FP8_E4M3 && !offs) return cudaErrorInvalidValue;
-    convert_uvw_kernel<<<grid_for(n_cells * 3 * D, 256), 256, 0, s>>>(in, out, n_cells, 3 * D, prec, rec_stride,
-                                                                        scales, offs, c0, k, oshift, odim, ostride);
+cudaError_t launch_convert_uvw(const float *in, char *out, int64_t r0, int64_t r1, int k, int D, int prec,
+                               int rec_stride, const float *scales, const uint16_t *offs, int oshift, int odim,
+                               int ostride, cudaStream_t s) {
+    if (r1 <= r0) return cudaSuccess;
+    constexpr int kSquare = 3;  // 8 x 8 rows per thread where no offset brick sets the square
+    if (prec == FNR_PREC_FP32)
+        convert_uvw_p<FNR_PREC_FP32>(in, out, r0, r1, k, 3 * D, rec_stride, scales, offs, kSquare, 0, 0, s);
+    else if (prec == FNR_PREC_FP16)
+        convert_uvw_p<FNR_PREC_FP16>(in, out, r0, r1, k, 3 * D, rec_stride, scales, offs, kSquare, 0, 0, s);
+    else if (!offs)
+        return cudaErrorInvalidValue;
+    else
+        convert_uvw_p<FNR_PREC_FP8_E4M3>(in, out, r0, r1, k, 3 * D, rec_stride, scales, offs, oshift, odim, ostride, s);
     return cudaGetLastError();
 }
 
-cudaError_t launch_brick_minmax(const float *uvw, int64_t c0, int64_t n, int k, int nch, int oshift, int odim,
+cudaError_t launch_brick_minmax(const float *uvw, int64_t r0, int64_t r1, int k, int nch, int oshift, int odim,
                                 unsigned *kmin, unsigned *kmax, cudaStream_t s) {
-    if (n <= 0) return cudaSuccess;
-    brick_minmax_kernel<<<grid_for(n, 256), 256, 0, s>>>(uvw, c0, n, k, nch, oshift, odim, kmin, kmax);
+    if (r1 <= r0) return cudaSuccess;
+    const int vec = group_width(uvw, static_cast<int64_t>(k) * nch);
+    int bz0;
+    const dim3 grid = row_grid(r0, r1, k, nch, vec, oshift, &bz0);
+    if (vec == 4)
+        brick_minmax_kernel<4><<<grid, kRowThreads, 0, s>>>(uvw, r0, r1, bz0, k, nch, oshift, odim, kmin, kmax);
+    else if (vec == 2)
+        brick_minmax_kernel<2><<<grid, kRowThreads, 0, s>>>(uvw, r0, r1, bz0, k, nch, oshift, odim, kmin, kmax);
+    else
+        brick_minmax_kernel<1><<<grid, kRowThreads, 0, s>>>(uvw, r0, r1, bz0, k, nch, oshift, odim, kmin, kmax);
     return cudaGetLastError();
 }
 
 cudaError_t launch_brick_offsets(const unsigned *kmin, const unsigned *kmax, int64_t n_bricks, int nch,
-                                 uint16_t *offs, int ostride, cudaStream_t s) {
+                                 uint16_t *offs, int ostride, unsigned *amax_bits, cudaStream_t s) {
     if (n_bricks <= 0) return cudaSuccess;
-    brick_offsets_kernel<<<grid_for(n_bricks * ostride, 256), 256, 0, s>>>(kmin, kmax, n_bricks, nch, offs, ostride);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_residual_absmax(const float *uvw, int64_t c0, int64_t n, int k, int nch, const uint16_t *offs,
-                                   int oshift, int odim, int ostride, unsigned *amax_bits, cudaStream_t s) {
-    if (n <= 0) return cudaSuccess;
-    residual_absmax_kernel<<<grid_for(n * nch, 256), 256, 0, s>>>(uvw, c0, n, k, nch, offs, oshift, odim, ostride,
-                                                                   amax_bits);
+    const int64_t blocks = std::min<int64_t>((n_bricks * ostride + 255) / 256, 152 * 8);
+    brick_offsets_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(kmin, kmax, n_bricks, nch, offs, ostride,
+                                                                        amax_bits);
     return cudaGetLastError();
 }
 
@@ -352,10 +552,10 @@ cudaError_t launch_convert_beta(const float *in, void *out, int64_t n, int prec,
     return cudaGetLastError();
 }
 
-cudaError_t launch_absmax(const float *sigma, const float *uvw, int64_t n_cells, int nch, unsigned *amax_bits,
-                          cudaStream_t s) {
-    if (n_cells <= 0) return cudaSuccess;
-    absmax_kernel<<<grid_for(n_cells * nch, 256), 256, 0, s>>>(sigma, uvw, n_cells, nch, amax_bits);
+cudaError_t launch_sigma_absmax(const float *sigma, int64_t n, unsigned *amax_bits, cudaStream_t s) {
+    if (n <= 0) return cudaSuccess;
+    if (aligned(sigma, 16)) sigma_absmax_kernel<4><<<grid_for((n + 3) / 4, 256), 256, 0, s>>>(sigma, n, amax_bits);
+    else sigma_absmax_kernel<1><<<grid_for(n, 256), 256, 0, s>>>(sigma, n, amax_bits);
     return cudaGetLastError();
 }
 
