@@ -106,8 +106,9 @@ static bool desc_valid(const fnr_cache_desc *d) {
 
 // Sections of one cache allocation. Dense: k^3 densities and records. Bricks
 // (n_bricks >= 0): pools of n_bricks * B^3 densities and records, then the
-// page table after the occupancy bits.
-static Layout layout_of(const fnr_cache_desc *d, int64_t n_bricks = -1) {
+// page table after the occupancy bits. Without records: a dense layout whose
+// record section is empty (the dense stage of a brick build from device arrays).
+static Layout layout_of(const fnr_cache_desc *d, int64_t n_bricks = -1, bool records = true) {
     Layout L;
     const bool bricks = d->layout == FNR_LAYOUT_BRICKS && n_bricks >= 0;
     const int sh = occupancy_shift(d);
@@ -118,7 +119,7 @@ static Layout layout_of(const fnr_cache_desc *d, int64_t n_bricks = -1) {
     L.off_sigma = off;
     off = align256(off + k3 * elem_bytes(d->pos_precision));
     L.off_uvw = off;
-    off = align256(off + k3 * uint64_t(L.rec_stride));
+    if (records) off = align256(off + k3 * uint64_t(L.rec_stride));
     L.off_beta = off;
     off = align256(off + uint64_t(d->l) * d->l * d->D * elem_bytes(d->dir_precision));
     L.off_ct = off;
@@ -183,7 +184,8 @@ struct DevBuf {
     }
 };
 
-static fnr_status build_from_arrays(fnr_cache *c, const fnr_cache_source *src, const Layout &L, cudaStream_t s) {
+static fnr_status build_from_arrays(fnr_cache *c, const fnr_cache_source *src, const Layout &L, bool records,
+                                    cudaStream_t s) {
     const fnr_cache_desc &d = c->desc;
     const int64_t k3 = int64_t(d.k) * d.k * d.k;
     const int nch = 3 * d.D;
@@ -253,7 +255,8 @@ static fnr_status build_from_arrays(fnr_cache *c, const fnr_cache_source *src, c
         if ((e = launch_convert_sigma(sp, base + L.off_sigma + c0 * elem_bytes(prec), n, prec, scales, s)) !=
             cudaSuccess)
             return cuda_fail(e, "density conversion");
-        if ((e = launch_convert_uvw(up, base + L.off_uvw + c0 * L.rec_stride, c0 / d.k, (c0 + n) / d.k, d.k, d.D, prec,
+        if (records &&
+            (e = launch_convert_uvw(up, base + L.off_uvw + c0 * L.rec_stride, c0 / d.k, (c0 + n) / d.k, d.k, d.D, prec,
                                     L.rec_stride, scales, offs, osh, odim, ostride, s)) != cudaSuccess)
             return cuda_fail(e, "uvw conversion");
         if (!dev && (e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "conversion sync");
@@ -451,30 +454,29 @@ uint64_t fnr_cache_footprint(const fnr_cache_desc *d) {
     return layout_of(d).total;
 }
 
+static fnr_status build_dense(fnr_context *ctx, const fnr_cache_desc *desc, const fnr_cache_source *src,
+                              bool records, cudaStream_t s, fnr_cache **out);
+
 // Dense cache -> FNR_LAYOUT_BRICKS cache: pool slots in brick-index order of
-// the occupied bricks, densities and records gathered brick by brick on the
-// GPU; the direction cache, tables, scales and occupancy bits are copied.
-static fnr_status make_bricks(fnr_context *ctx, const fnr_cache *dense, const fnr_cache_desc *desc,
-                              cudaStream_t s, fnr_cache **out) {
+// the occupied bricks, found on the GPU (only their count is read back, for the
+// allocation); the densities are gathered brick by brick, and so are the records,
+// or converted straight from the binary32 source `uvw` if the dense stage has
+// none; the direction cache, tables, scales and occupancy bits are copied.
+static fnr_status make_bricks(fnr_context *ctx, const fnr_cache *dense, const Layout &LD, const float *uvw,
+                              const fnr_cache_desc *desc, cudaStream_t s, fnr_cache **out) {
     const CacheView &dv = dense->view;
-    const int64_t nb = dv.occ_dim, nb3 = nb * nb * nb;
-    std::vector<uint32_t> words(occupancy_words(desc));
+    const int64_t nb = dv.occ_dim, nb3 = nb * nb * nb, n_words = int64_t(occupancy_words(desc));
     cudaError_t e;
-    if ((e = cudaMemcpyAsync(words.data(), dv.occ, words.size() * 4, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+    DevBuf rank;
+    uint32_t total = 0;
+    if ((e = dev_malloc(&rank.p, size_t(n_words + 1) * 4)) != cudaSuccess) return cuda_fail(e, "brick ranks");
+    uint32_t *rk = static_cast<uint32_t *>(rank.p);
+    if ((e = launch_brick_rank(dv.occ, n_words, rk, rk + n_words, s)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(&total, rk + n_words, 4, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
         (e = cudaStreamSynchronize(s)) != cudaSuccess)
-        return cuda_fail(e, "occupancy read-back");
-    std::vector<int32_t> page(size_t(nb3), -1), slot_brick;
-    std::vector<uint32_t> rank(words.size());
-    for (int64_t b = 0; b < nb3; ++b) {
-        if ((b & 31) == 0) rank[size_t(b >> 5)] = uint32_t(slot_brick.size());
-        if ((words[size_t(b >> 5)] >> (b & 31)) & 1u) {
-            page[size_t(b)] = int32_t(slot_brick.size());
-            slot_brick.push_back(int32_t(b));
-        }
-    }
-    const int64_t n_bricks = int64_t(slot_brick.size());
+        return cuda_fail(e, "brick count");
+    const int64_t n_bricks = total;
     const Layout L = layout_of(desc, n_bricks);
-    const Layout LD = layout_of(&dense->desc);
     if (!budget_charge(ctx, L.total))
         return fail(FNR_ERR_BUDGET, "brick cache needs %llu bytes, budget %llu, in use %llu",
                     (unsigned long long)L.total, (unsigned long long)ctx->budget,
@@ -493,24 +495,29 @@ static fnr_status make_bricks(fnr_context *ctx, const fnr_cache *dense, const fn
     const char *dbase = static_cast<const char *>(dense->base);
     DevBuf slots;
     fnr_status st = FNR_OK;
-    if (n_bricks > 0 && (e = dev_malloc(&slots.p, size_t(n_bricks) * 4)) != cudaSuccess) st = cuda_fail(e, "slots");
+    if ((e = dev_malloc(&slots.p, size_t(std::max<int64_t>(n_bricks, 1)) * 4)) != cudaSuccess) st = cuda_fail(e, "slots");
+    const int32_t *sb = static_cast<const int32_t *>(slots.p);
     if (st == FNR_OK &&
-        ((n_bricks > 0 && (e = cudaMemcpyAsync(slots.p, slot_brick.data(), size_t(n_bricks) * 4,
-                                               cudaMemcpyHostToDevice, s)) != cudaSuccess) ||
-         (e = cudaMemcpyAsync(base + L.off_page, page.data(), size_t(nb3) * 4, cudaMemcpyHostToDevice, s)) !=
-             cudaSuccess ||
-         (e = cudaMemcpyAsync(base + L.off_rank, rank.data(), rank.size() * 4, cudaMemcpyHostToDevice, s)) !=
+        ((e = launch_brick_pages(dv.occ, rk, nb3, reinterpret_cast<int32_t *>(base + L.off_page),
+                                 static_cast<int32_t *>(slots.p), s)) != cudaSuccess ||
+         (e = cudaMemcpyAsync(base + L.off_rank, rk, size_t(n_words) * 4, cudaMemcpyDeviceToDevice, s)) !=
              cudaSuccess ||
          (e = cudaMemcpyAsync(base + L.off_beta, dbase + LD.off_beta, L.off_page - L.off_beta,
                               cudaMemcpyDeviceToDevice, s)) != cudaSuccess))
         st = cuda_fail(e, "brick cache tables");
     // (beta, the bin tables, the scales, the occupancy bits and the brick distances keep their
     // relative offsets)
-    if (st == FNR_OK && n_bricks > 0 &&
-        (e = launch_gather_bricks(dv.sigma, dv.uvw, base + L.off_sigma, base + L.off_uvw,
-                                  static_cast<const int32_t *>(slots.p), n_bricks, desc->k, dv.occ_shift,
-                                  dv.occ_dim, int(elem_bytes(desc->pos_precision)), L.rec_stride, s)) != cudaSuccess)
-        st = cuda_fail(e, "brick gather");
+    if (st == FNR_OK && n_bricks > 0) {
+        e = launch_gather_bricks(dv.sigma, base + L.off_sigma, sb, n_bricks, desc->k, dv.occ_shift, dv.occ_dim,
+                                 int(elem_bytes(desc->pos_precision)), s);
+        if (e == cudaSuccess)
+            e = uvw ? launch_convert_bricks(uvw, base + L.off_uvw, sb, n_bricks, desc->k, desc->D, desc->pos_precision,
+                                            L.rec_stride, dv.occ_shift, dv.occ_dim, dv.scales, dv.offs, dv.offs_shift,
+                                            dv.offs_dim, dv.offs_stride, s)
+                    : launch_gather_bricks(dv.uvw, base + L.off_uvw, sb, n_bricks, desc->k, dv.occ_shift, dv.occ_dim,
+                                           L.rec_stride, s);
+        if (e != cudaSuccess) st = cuda_fail(e, "brick gather");
+    }
     if (st == FNR_OK && (e = cudaStreamSynchronize(s)) != cudaSuccess) st = cuda_fail(e, "brick cache sync");
     if (st != FNR_OK) {
         cudaFree(c->base);
@@ -534,18 +541,27 @@ fnr_status fnr_build_cache(fnr_context *ctx, const fnr_cache_desc *desc, const f
     if (!ctx || !desc || !src || !out) return fail(FNR_ERR_INVALID_ARG, "NULL argument");
     *out = nullptr;
     if (!desc_valid(desc)) return fail(FNR_ERR_INVALID_ARG, "invalid cache descriptor");
-    if (desc->layout == FNR_LAYOUT_BRICKS) {  // through a dense cache, freed afterwards
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    if (desc->layout == FNR_LAYOUT_BRICKS) {
+        // through a dense stage, freed afterwards and charged as a dense cache while it exists; the records of
+        // device arrays are converted brick by brick, so that stage then holds none
         fnr_cache_desc dd = *desc;
         dd.layout = FNR_LAYOUT_DENSE;
+        const bool direct = src->kind == FNR_SRC_ARRAYS && src->location == FNR_LOC_DEVICE;
         fnr_cache *dense = nullptr;
-        fnr_status st = fnr_build_cache(ctx, &dd, src, stream, &dense);
+        fnr_status st = build_dense(ctx, &dd, src, !direct, s, &dense);
         if (st != FNR_OK) return st;
-        st = make_bricks(ctx, dense, desc, reinterpret_cast<cudaStream_t>(stream), out);
+        st = make_bricks(ctx, dense, layout_of(&dd, -1, !direct), direct ? src->uvw : nullptr, desc, s, out);
         std::string msg = st != FNR_OK ? std::string(fnr_last_error()) : std::string();
         fnr_cache_free(ctx, dense);
         if (st != FNR_OK) return fail(st, "%s", msg.c_str());
         return FNR_OK;
     }
+    return build_dense(ctx, desc, src, true, s, out);
+}
+
+static fnr_status build_dense(fnr_context *ctx, const fnr_cache_desc *desc, const fnr_cache_source *src,
+                              bool records, cudaStream_t s, fnr_cache **out) {
     fnr_status st0;
     if (src->kind == FNR_SRC_MLP) {
         if ((st0 = check_mlp(src->pos_mlp, 1 + 3 * desc->D, "pos_mlp")) != FNR_OK) return st0;
@@ -561,20 +577,20 @@ fnr_status fnr_build_cache(fnr_context *ctx, const fnr_cache_desc *desc, const f
     }
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_fail(e, "cudaSetDevice");
-    const Layout L = layout_of(desc);
-    if (!budget_charge(ctx, L.total))
-        return fail(FNR_ERR_BUDGET, "cache needs %llu bytes, budget %llu, in use %llu", (unsigned long long)L.total,
+    const Layout L = layout_of(desc, -1, records);
+    const uint64_t charge = layout_of(desc).total;
+    if (!budget_charge(ctx, charge))
+        return fail(FNR_ERR_BUDGET, "cache needs %llu bytes, budget %llu, in use %llu", (unsigned long long)charge,
                     (unsigned long long)ctx->budget, (unsigned long long)ctx->used.load());
     fnr_cache *c = new fnr_cache();
     c->desc = *desc;
-    c->footprint = L.total;
+    c->footprint = charge;
     c->ctx = ctx;
     if ((e = dev_malloc(&c->base, L.total)) != cudaSuccess) {
-        budget_uncharge(ctx, L.total);
+        budget_uncharge(ctx, charge);
         delete c;
         return cuda_fail(e, "cache allocation");
     }
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     std::vector<float> ct, qp;
     bin_tables(desc->l, ct, qp);
     char *base = static_cast<char *>(c->base);
@@ -593,7 +609,7 @@ fnr_status fnr_build_cache(fnr_context *ctx, const fnr_cache_desc *desc, const f
     }
     if (st == FNR_OK) {
         if (src->kind == FNR_SRC_ARRAYS) {
-            st = build_from_arrays(c, src, L, s);
+            st = build_from_arrays(c, src, L, records, s);
         } else {
             fill_view(c, L);
             st = run_mlp(src->pos_mlp, 0, c->desc, c->view, ctx->num_sms, s);
@@ -613,7 +629,7 @@ fnr_status fnr_build_cache(fnr_context *ctx, const fnr_cache_desc *desc, const f
     }
     if (st != FNR_OK) {
         cudaFree(c->base);
-        budget_uncharge(ctx, L.total);
+        budget_uncharge(ctx, charge);
         delete c;
         return st;
     }

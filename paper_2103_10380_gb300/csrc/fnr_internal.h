@@ -119,10 +119,19 @@ size_t elem_bytes(int prec);
 
 // Launchers (march.cu / quant.cu). Return cudaError_t of the launch.
 cudaError_t launch_march(const MarchArgs &a, cudaStream_t s);
-// Dense cache -> brick pools: pool slot s holds brick slot_brick[s] (k^3 grid, bricks of 2^shift cells).
-cudaError_t launch_gather_bricks(const void *sigma, const char *uvw, void *sigma_pool, char *uvw_pool,
-                                 const int32_t *slot_brick, int64_t n_bricks, int k, int shift, int dim,
-                                 int s_sigma, int rec_stride, cudaStream_t s);
+// Brick pools. rank[w] = set occupancy bits of the words before w, *total = all of them; then page[b] =
+// slot or -1 and slot_brick[slot] = b over the bricks in index order.
+cudaError_t launch_brick_rank(const uint32_t *words, int64_t n_words, uint32_t *rank, uint32_t *total,
+                              cudaStream_t s);
+cudaError_t launch_brick_pages(const uint32_t *words, const uint32_t *rank, int64_t n_bricks, int32_t *page,
+                               int32_t *slot_brick, cudaStream_t s);
+// Pool slot s gets the cells of brick slot_brick[s] (k^3 grid, bricks of 2^shift cells, dim per axis) of a
+// dense plane of `stride` bytes per cell; or the records of those cells straight from the binary32 source.
+cudaError_t launch_gather_bricks(const void *plane, void *pool, const int32_t *slot_brick, int64_t n_bricks, int k,
+                                 int shift, int dim, int stride, cudaStream_t s);
+cudaError_t launch_convert_bricks(const float *uvw, char *pool, const int32_t *slot_brick, int64_t n_bricks, int k,
+                                  int D, int prec, int rec_stride, int shift, int dim, const float *scales,
+                                  const uint16_t *offs, int oshift, int odim, int ostride, cudaStream_t s);
 cudaError_t launch_convert_sigma(const float *in, void *out, int64_t n, int prec, const float *scale,
                                  cudaStream_t s);
 // The records of the x-rows [r0, r1) (row z k + y; `in` and `out` point at row r0).
