@@ -261,3 +261,33 @@ def test_cta_pair_form_bit_identical(fnr, k, l, pos_dims, dir_dims):
     finally:
         fnr.fnr_testing_mlp_cta_pair(False)
         fnr.fnr_context_destroy(ctx)
+
+
+@pytest.mark.parametrize("k,l,D,pos_dims,dir_dims", [
+    (37, 300, 8, scenegen.FPOS_DIMS_D8, scenegen.FDIR_DIMS_D8),          # a last pair of one tile; narrow, many rounds
+    (30, 150, 16, [60, 256, 49], [60, 16]),                              # two passes of a head; one layer
+    (20, 200, 4, [60, 144, 200, 64, 16, 25], [24, 16, 8]),               # halves of 16 and 72 outputs, padded inputs
+    (11, 9, 8, [60] + [256] * 15 + [25], [64, 256, 256, 30]),            # the deepest network; outputs not stored
+    (70, 20, 2, [24, 128, 129, 128, 7], [24, 32, 2]),                    # widths at a half's edge
+])
+def test_forms_agree_over_shapes(fnr, k, l, D, pos_dims, dir_dims):
+    """The single-CTA form (activations in tensor memory, outputs in halves of 128) against the CTA-pair form
+    (activations in shared memory, all outputs at once), both accumulating each output over the inputs in the
+    same order: caches equal byte for byte."""
+    pos = to_device(scenegen.mlp_weights(17, pos_dims, bias_scale=0.3))
+    dirn = to_device(scenegen.mlp_weights(18, dir_dims, bias_scale=0.3))
+    pos_freqs, dir_freqs = pos_dims[0] // 6, min(dir_dims[0] // 6, 10)
+    ctx = fnr.fnr_context_create(0, 0)
+    try:
+        for prec in (fnr.FNR_PREC_FP32, fnr.FNR_PREC_FP16):
+            outs = []
+            for pair in (True, False):
+                fnr.fnr_testing_mlp_cta_pair(pair)
+                c = fnr.fnr_build_cache_mlp(ctx, fnr.make_desc(k, D, l, prec, prec), pos, dirn, pos_freqs, dir_freqs)
+                outs.append(read_cache(fnr, c, k, D, l, prec, prec))
+                fnr.fnr_cache_free(ctx, c)
+            for a, b in zip(*outs):
+                assert np.array_equal(a, b)
+    finally:
+        fnr.fnr_testing_mlp_cta_pair(False)
+        fnr.fnr_context_destroy(ctx)
