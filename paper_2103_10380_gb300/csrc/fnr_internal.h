@@ -169,8 +169,21 @@ void server_stop(fnr_context *ctx);
 
 // mlp.cu: tensor-core evaluation of F_pos (mode 0) / F_dir (mode 1) into a cache.
 fnr_status check_mlp(const fnr_mlp *m, int n_out_min, const char *name);
-fnr_status run_mlp_points(const fnr_mlp *m, const float *points, long long n, float *out, int out_stride,
-                          bool relu0, int num_sms, cudaStream_t s);
+// The same at listed points: prepare() lays the weights out once, each launch() evaluates [n][3] points on the
+// device (n read from n_dev, at most max_n; n = max_n if n_dev is null), the first out_stride head outputs of
+// point p going to out[p * out_stride + c] in FP32 (channel 0 through ReLU if relu0), finish() waits and reports.
+class PointsMlp {
+public:
+    ~PointsMlp();
+    fnr_status prepare(const fnr_mlp *m, int out_stride, bool relu0, cudaStream_t s);
+    fnr_status launch(const float *points, long long max_n, const unsigned long long *n_dev, float *out, int num_sms,
+                      cudaStream_t s);
+    fnr_status finish(cudaStream_t s);
+
+private:
+    struct Impl;
+    Impl *impl = nullptr;
+};
 fnr_status run_mlp(const fnr_mlp *m, int mode, const fnr_cache_desc &d, const CacheView &v, int num_sms,
                    cudaStream_t s);
 

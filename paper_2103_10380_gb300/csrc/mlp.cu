@@ -265,7 +265,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_kernel(const __grid_constant_
     const uint32_t tmem = *tmem_slot;
     // Tiles go to CTAs in pairs: pair r of CTA b holds tiles (2 r + t) * grid + b. The last pair may
     // hold one.
-    const int n_tiles = A.n_tiles, G = int(gridDim.x), bid = int(blockIdx.x);
+    const long long n_points = point_count(A);
+    const int n_tiles = int((n_points + kTileM - 1) / kTileM), G = int(gridDim.x), bid = int(blockIdx.x);
     auto tile_of = [&](int r, int t) { return (kPair * r + t) * G + bid; };
     auto tiles_in = [&](int r) { return tile_of(r, 1) < n_tiles ? 2 : 1; };
     const int n_pairs = n_tiles > bid ? (n_tiles - bid + kPair * G - 1) / (kPair * G) : 0;
@@ -334,7 +335,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_kernel(const __grid_constant_
         auto encode = [&](int r, int t) {
             // pair r - 1's layer-0 MMAs have read the buffer
             if (r > 0 && !warp_wait(enc_free(t), uint32_t((r - 1) & 1))) return false;
-            encode_point(A, (long long)tile_of(r, t) * kTileM + q * 32 + lane, q * 32 + lane, stage + size_t(t) * kStageBytes);
+            encode_point(A, n_points, (long long)tile_of(r, t) * kTileM + q * 32 + lane, q * 32 + lane,
+                         stage + size_t(t) * kStageBytes);
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(enc_ready(t));
@@ -345,7 +347,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_kernel(const __grid_constant_
             if (!warp_wait(head_full(t), uint32_t(r & 1))) return false;
             tc_fence_after();
             const long long p0 = (long long)tile_of(r, t) * kTileM + q * 32;
-            const int nv = int(A.n_points - p0 < 32 ? (A.n_points > p0 ? A.n_points - p0 : 0) : 32);
+            const int nv = int(n_points - p0 < 32 ? (n_points > p0 ? n_points - p0 : 0) : 32);
 #pragma unroll 1
             for (int c0 = 0; c0 < n; c0 += kHeadCols) {  // 32 outputs at a time
                 const int nc = min(n - c0, kHeadCols);
@@ -590,12 +592,11 @@ fnr_status launch_mlp_single(const MlpArgs &A, int num_sms, cudaStream_t s) {
     cudaError_t e;
     // tile indices, one pair per CTA past the end included, are int
     if (A.n_points > (1LL << 37)) return fail(FNR_ERR_UNSUPPORTED, "MLP kernel: %lld points", A.n_points);
-    MlpArgs B = A;
-    B.n_tiles = int((A.n_points + kTileM - 1) / kTileM);
+    const int tiles = int((A.n_points + kTileM - 1) / kTileM);
     if ((e = cudaFuncSetAttribute(mlp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemBytes))) !=
         cudaSuccess)
         return cuda_fail(e, "MLP smem attribute");
-    mlp_kernel<<<unsigned(B.n_tiles < num_sms ? B.n_tiles : num_sms), kThreads, kSmemBytes, s>>>(B);
+    mlp_kernel<<<unsigned(tiles < num_sms ? tiles : num_sms), kThreads, kSmemBytes, s>>>(A);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "MLP launch");
     return FNR_OK;
 }
@@ -623,25 +624,28 @@ fnr_status check_mlp(const fnr_mlp *m, int n_out_min, const char *name) {
 
 namespace {
 
-// Lay out the weights and biases of m, fill the layer table of A, launch the
-// kernel on the mode-specific arguments already in A, and wait for it.
-fnr_status mlp_launch(const fnr_mlp *m, MlpArgs &A, int num_sms, cudaStream_t s) {
-    struct Buf {
-        void *p = nullptr;
-        ~Buf() {
-            if (p) cudaFree(p);
-        }
-    } wbuf, bbuf, ebuf;
+// Device copies of one network's weights and biases, and the error word of its launches.
+struct MlpBuffers {
+    void *weights = nullptr, *biases = nullptr, *err = nullptr;
+    ~MlpBuffers() {
+        if (weights) cudaFree(weights);
+        if (biases) cudaFree(biases);
+        if (err) cudaFree(err);
+    }
+};
+
+// Lay out the weights and biases of m and fill the layer table of A (A.mode and its outputs per point are set).
+fnr_status mlp_prepare(const fnr_mlp *m, MlpArgs &A, MlpBuffers &B, cudaStream_t s) {
     size_t welems = 0, belems = 0;
     for (int i = 0; i < m->n_layers; ++i) {
         welems += size_t(round16(m->dims[i + 1])) * round64(m->dims[i]);
         belems += size_t(round16(m->dims[i + 1]));
     }
     cudaError_t e;
-    if ((e = dev_malloc(&wbuf.p, welems * 2)) != cudaSuccess) return cuda_fail(e, "MLP weights");
-    if ((e = dev_malloc(&bbuf.p, belems * 4)) != cudaSuccess) return cuda_fail(e, "MLP biases");
-    if ((e = dev_malloc(&ebuf.p, 4)) != cudaSuccess) return cuda_fail(e, "MLP error word");
-    if ((e = cudaMemsetAsync(ebuf.p, 0, 4, s)) != cudaSuccess) return cuda_fail(e, "memset");
+    if ((e = dev_malloc(&B.weights, welems * 2)) != cudaSuccess) return cuda_fail(e, "MLP weights");
+    if ((e = dev_malloc(&B.biases, belems * 4)) != cudaSuccess) return cuda_fail(e, "MLP biases");
+    if ((e = dev_malloc(&B.err, 4)) != cudaSuccess) return cuda_fail(e, "MLP error word");
+    if ((e = cudaMemsetAsync(B.err, 0, 4, s)) != cudaSuccess) return cuda_fail(e, "memset");
     A.n_out = A.mode == 0 ? 1 + 3 * A.D : (A.mode == 1 ? A.D : A.out_stride);
     if (A.n_out < 1 || A.n_out > kMaxOut || A.n_out > m->dims[m->n_layers])
         return fail(FNR_ERR_UNSUPPORTED, "MLP kernel: %d outputs per point (at most %d)", A.n_out, kMaxOut);
@@ -652,11 +656,11 @@ fnr_status mlp_launch(const fnr_mlp *m, MlpArgs &A, int num_sms, cudaStream_t s)
     for (int i = 0; i < m->n_layers; ++i) {
         // the head is evaluated up to the outputs that are stored
         const int K = m->dims[i], N = i + 1 == m->n_layers ? A.n_out : m->dims[i + 1], Kp = round64(K), Np = round16(N);
-        uint16_t *wd = static_cast<uint16_t *>(wbuf.p) + wo;
+        uint16_t *wd = static_cast<uint16_t *>(B.weights) + wo;
         P.w[i] = m->weights[i];
         P.b[i] = m->biases[i];
         P.w_out[i] = wd;
-        P.b_out[i] = static_cast<float *>(bbuf.p) + bo;
+        P.b_out[i] = static_cast<float *>(B.biases) + bo;
         P.N[i] = N;
         P.K[i] = K;
         P.Np[i] = Np;
@@ -671,19 +675,28 @@ fnr_status mlp_launch(const fnr_mlp *m, MlpArgs &A, int num_sms, cudaStream_t s)
     }
     prepare_kernel<<<dim3(unsigned((max_elems + 255) / 256), unsigned(m->n_layers)), 256, 0, s>>>(P);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "MLP weight layout");
-    A.bias = static_cast<const float *>(bbuf.p);
+    A.bias = static_cast<const float *>(B.biases);
     A.n_bias = int(bo);
     A.n_layers = m->n_layers;
     A.pe_freqs = m->pe_freqs;
-    A.err = static_cast<int *>(ebuf.p);
+    A.err = static_cast<int *>(B.err);
     A.wait_limit = kWaitLimit;
     A.withhold = -1;
     take_mlp_fault(&A.wait_limit, &A.withhold);
+    return FNR_OK;
+}
+
+// One launch over the points already in A.
+fnr_status mlp_launch(const MlpArgs &A, int num_sms, cudaStream_t s) {
     if (A.n_points <= 0) return FNR_OK;
-    const fnr_status st = mlp_cta_pair() ? launch_mlp_pair(A, num_sms, s) : launch_mlp_single(A, num_sms, s);
-    if (st != FNR_OK) return st;
+    return mlp_cta_pair() ? launch_mlp_pair(A, num_sms, s) : launch_mlp_single(A, num_sms, s);
+}
+
+// Wait for the launches on A and report their error word.
+fnr_status mlp_finish(const MlpArgs &A, cudaStream_t s) {
     int herr = 0;
-    if ((e = cudaMemcpyAsync(&herr, ebuf.p, 4, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+    cudaError_t e;
+    if ((e = cudaMemcpyAsync(&herr, A.err, 4, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
         (e = cudaStreamSynchronize(s)) != cudaSuccess)
         return cuda_fail(e, "MLP sync");
     if (herr == 1) return fail(FNR_ERR_DEVICE, "MLP kernel: an mbarrier wait ran out");
@@ -713,22 +726,38 @@ fnr_status run_mlp(const fnr_mlp *m, int mode, const fnr_cache_desc &d, const Ca
     A.D = d.D;
     A.beta_out = const_cast<void *>(v.beta);
     A.dprec = d.dir_precision;
-    return mlp_launch(m, A, num_sms, s);
+    MlpBuffers B;
+    fnr_status st = mlp_prepare(m, A, B, s);
+    if (st == FNR_OK) st = mlp_launch(A, num_sms, s);
+    return st == FNR_OK ? mlp_finish(A, s) : st;
 }
 
-// Evaluate one MLP at n listed points ([n][3] on the device): the first
-// out_stride head outputs of point p go to out[p * out_stride + c] in FP32.
-fnr_status run_mlp_points(const fnr_mlp *m, const float *points, long long n, float *out, int out_stride,
-                          bool relu0, int num_sms, cudaStream_t s) {
+struct PointsMlp::Impl {
     MlpArgs A;
-    memset(&A, 0, sizeof(A));
-    A.mode = 2;
-    A.n_points = n;
+    MlpBuffers B;
+};
+
+PointsMlp::~PointsMlp() { delete impl; }
+
+fnr_status PointsMlp::prepare(const fnr_mlp *m, int out_stride, bool relu0, cudaStream_t s) {
+    impl = new Impl();
+    memset(&impl->A, 0, sizeof(impl->A));
+    impl->A.mode = 2;
+    impl->A.out_stride = out_stride;
+    impl->A.relu0 = relu0 ? 1 : 0;
+    return mlp_prepare(m, impl->A, impl->B, s);
+}
+
+fnr_status PointsMlp::launch(const float *points, long long max_n, const unsigned long long *n_dev, float *out,
+                             int num_sms, cudaStream_t s) {
+    MlpArgs A = impl->A;
+    A.n_points = max_n;
+    A.n_dev = n_dev;
     A.points = points;
     A.out = out;
-    A.out_stride = out_stride;
-    A.relu0 = relu0 ? 1 : 0;
-    return mlp_launch(m, A, num_sms, s);
+    return mlp_launch(A, num_sms, s);
 }
+
+fnr_status PointsMlp::finish(cudaStream_t s) { return mlp_finish(impl->A, s); }
 
 }  // namespace fnr

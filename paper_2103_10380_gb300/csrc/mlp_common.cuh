@@ -39,8 +39,8 @@ struct MlpArgs {
     int pe_freqs;
     int k, l;
     float bmin[3], h[3];
-    long long n_points;
-    int n_tiles;     // MMA tiles of kTileM points (single-CTA form)
+    long long n_points;                // or, with n_dev, their upper bound
+    const unsigned long long *n_dev;   // the number of points, if the host does not know it
     // outputs
     void *sigma_out;   // mode 0
     char *uvw_out;     // mode 0
@@ -197,14 +197,18 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     return uint32_t(__bfloat16_as_ushort(x)) | (uint32_t(__bfloat16_as_ushort(y)) << 16);
 }
 
+__device__ __forceinline__ long long point_count(const MlpArgs &A) {
+    return A.n_dev ? static_cast<long long>(*A.n_dev) : A.n_points;
+}
+
 // Positional encoding of point p into row `row` of a layer-0 A tile (K0 <= 64
 // columns, one 128-byte swizzled row): column 2 P + 0 / 1 holds sin / cos(2^j
 // pi x_a) with P = a L + j, rounded to bf16; columns from 6 L on, and every
 // column of a point past the end, are 0.
-__device__ __forceinline__ void encode_point(const MlpArgs &A, long long p, int row, char *sa) {
+__device__ __forceinline__ void encode_point(const MlpArgs &A, long long n_points, long long p, int row, char *sa) {
     const int K0 = A.L[0].K;
     float x0 = 0.0f, x1 = 0.0f, x2 = 0.0f;
-    const bool valid = p < A.n_points;
+    const bool valid = p < n_points;
     if (valid) {
         if (A.mode == 2) {
             x0 = A.points[3 * p];

@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_pair_kernel(const __grid_cons
     // MMA tiles of kSuperM points go to CTAs (pairs) in groups of kPair: group r holds tiles
     // (kPair r + t) * grid + bid, t < kPair; a tile past the end is carried as an empty one (no outputs).
     // CTA `rank` of a pair holds rows [rank kTileM, rank kTileM + kTileM) of each tile.
-    const long long n_tiles = (A.n_points + kSuperM - 1) / kSuperM;
+    const long long n_points = point_count(A), n_tiles = (n_points + kSuperM - 1) / kSuperM;
     const long long G = gridDim.x / kCtas;
     const long long bid = blockIdx.x / kCtas;
     auto pair_tile = [&](long long r, int t) { return (kPair * r + t) * G + bid; };
@@ -316,8 +316,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_pair_kernel(const __grid_cons
                 char *st = stage + size_t(t) * kStageBytes;
                 for (int row = e * 32 + lane; row < kTileM; row += 32 * kEncWarps) {
                     const long long p =
-                        tile < n_tiles ? tile * kSuperM + rank * kTileM + row : A.n_points;  // past the end: zeros
-                    encode_point(A, p, row, st);
+                        tile < n_tiles ? tile * kSuperM + rank * kTileM + row : n_points;  // past the end: zeros
+                    encode_point(A, n_points, p, row, st);
                 }
                 fence_proxy_async();
                 __syncwarp();
@@ -414,8 +414,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_pair_kernel(const __grid_cons
                     // element e of the range belongs to row e / n and output e % n
                     const long long tile = pair_tile(r, t);
                     const long long p0 = tile * kSuperM + rank * kTileM;
-                    const int nv = tile < n_tiles && p0 < A.n_points
-                                       ? int(A.n_points - p0 < kTileM ? A.n_points - p0 : kTileM)
+                    const int nv = tile < n_tiles && p0 < n_points
+                                       ? int(n_points - p0 < kTileM ? n_points - p0 : kTileM)
                                        : 0;
                     constexpr int kEpiThreads = 32 * kEpiWarps;
                     if (A.mode == 0) {

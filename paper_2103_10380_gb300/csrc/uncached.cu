@@ -2,13 +2,21 @@
 // box and F_dir per ray, evaluated by the tensor-core MLP kernel (mlp.cu), then
 // composited with Eq. 5 and Eq. 1 exactly as the cached march does.
 //
-//   samples_kernel: per ray, the inside samples' positions into one compact
-//     list (a warp-aggregated atomic hands each ray its range) and the ray's
-//     unit direction;
-//   F_pos over the list, F_dir over the directions (run_mlp_points);
+//   directions_kernel: every ray's unit direction, and F_dir over them;
+//   then, batch by batch of rays (at most 8 Mi samples):
+//   samples_kernel: the inside samples' positions in one compact list (a
+//     warp-aggregated atomic hands each ray its range);
+//   F_pos over the list (PointsMlp; its length stays on the device);
 //   composite_kernel: per ray, beta from F_dir, then the samples in order:
 //     sigma and (u, v, w) from F_pos, Eq. 5 + activation, Eq. 1 and the exact
 //     integer termination; RGBA and counters.
+// The networks' FLOPs are what the call cannot do without. The batches keep
+// the temporaries at one GB and nothing waits between them: an 800 x 800 view of
+// 128 samples has 9 GB of them in one piece, whose allocation and release and
+// whose wait for the number of samples took 5 of 45 ms. Batches of 2 / 4 / 8 Mi
+// samples: 44.0 / 40.6 / 39.0 ms (each launch has its ramp and its last wave).
+#include <algorithm>
+
 #include "march_device.cuh"
 #include "nvtx_range.h"
 
@@ -65,54 +73,70 @@ __device__ __forceinline__ bool sample_at(const Ray &r, const RenderConst &rc, c
     return in;
 }
 
-__global__ void samples_kernel(const FrameDesc F, const RenderConst rc, const Box b, float *points,
-                               unsigned long long *total, long long *offset, int *count, float *dirs) {
+__global__ void directions_kernel(const FrameDesc F, float *dirs) {
     const int ray = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n_rays = F.W * F.H;
-    const bool active = ray < n_rays;
-    Ray r;
-    int n = 0;
-    if (active) {
-        r = make_ray(F, ray % F.W, ray / F.W);
-        float p[3];
-        for (int i = 0; i < rc.N; ++i) n += sample_at(r, rc, b, i, p) ? 1 : 0;
-    }
-    // one atomic per warp for the warp's rays
-    const unsigned full = __activemask();
-    int incl = n;
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int dd = 1; dd < 32; dd <<= 1) {
-        const int v = __shfl_up_sync(full, incl, dd);
-        if (lane >= dd) incl += v;
-    }
-    const int last = 31 - __clz(full);
-    unsigned long long base = 0;
-    if (lane == last) base = atomicAdd(total, static_cast<unsigned long long>(incl));
-    base = __shfl_sync(full, base, last);
-    if (!active) return;
-    const long long off = static_cast<long long>(base) + incl - n;
-    offset[ray] = off;
-    count[ray] = n;
+    if (ray >= F.W * F.H) return;
+    const Ray r = make_ray(F, ray % F.W, ray / F.W);
     dirs[3 * ray] = r.d[0];
     dirs[3 * ray + 1] = r.d[1];
     dirs[3 * ray + 2] = r.d[2];
-    long long j = off;
-    float p[3];
-    for (int i = 0; i < rc.N; ++i)
-        if (sample_at(r, rc, b, i, p)) {
-            points[3 * j] = p[0];
-            points[3 * j + 1] = p[1];
-            points[3 * j + 2] = p[2];
-            ++j;
+}
+
+// Rays [ray0, ray0 + n_rays). A ray's inside samples are consecutive (t_i, and so each coordinate, is monotone in
+// i), so a lane finds its ray's first and their number, and the warp writes the rays' positions one ray after the
+// other, 32 samples at a time (a lane writing its own ray's scattered them: 328 us for 400 x 400 rays of 128).
+__global__ void samples_kernel(const FrameDesc F, const RenderConst rc, const Box b, int ray0, int n_rays,
+                               float *points, unsigned long long *total, long long *offset) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int i_ray = blockIdx.x * blockDim.x + threadIdx.x, ray = ray0 + i_ray, lane = threadIdx.x & 31;
+    const bool active = i_ray < n_rays;
+    Ray r = {};
+    int first = 0, n = 0;
+    if (active) {
+        r = make_ray(F, ray % F.W, ray / F.W);
+        float p[3];
+        for (int i = rc.N - 1; i >= 0; --i)
+            if (sample_at(r, rc, b, i, p)) {
+                first = i;
+                ++n;
+            }
+    }
+    // one atomic per warp for the warp's rays
+    int incl = n;
+#pragma unroll
+    for (int dd = 1; dd < 32; dd <<= 1) {
+        const int v = __shfl_up_sync(FULL, incl, dd);
+        if (lane >= dd) incl += v;
+    }
+    unsigned long long base = 0;
+    if (lane == 31) base = atomicAdd(total, static_cast<unsigned long long>(incl));
+    base = __shfl_sync(FULL, base, 31);
+    if (active) offset[i_ray] = static_cast<long long>(base) + incl - n;
+    float *out = points + 3 * base;
+    for (int j = 0; j < 32; ++j) {
+        const int nj = __shfl_sync(FULL, n, j), fj = __shfl_sync(FULL, first, j);
+        Ray q;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            q.d[a] = __shfl_sync(FULL, r.d[a], j);
+            q.o[a] = F.c2w[4 * a + 3];
         }
+        for (int i = lane; i < nj; i += 32) {
+            float p[3];
+            sample_at(q, rc, b, fj + i, p);
+            out[3 * i] = p[0];
+            out[3 * i + 1] = p[1];
+            out[3 * i + 2] = p[2];
+        }
+        out += 3 * nj;
+    }
 }
 
 template <int D>
-__global__ void composite_kernel(const FrameDesc F, const RenderConst rc, const Box b, const float *pos_out,
-                                 const float *dir_out, const long long *offset) {
-    const int ray = blockIdx.x * blockDim.x + threadIdx.x;
-    if (ray >= F.W * F.H) return;
+__global__ void composite_kernel(const FrameDesc F, const RenderConst rc, const Box b, int ray0, int n_rays,
+                                 const float *pos_out, const float *dir_out, const long long *offset) {
+    const int i_ray = blockIdx.x * blockDim.x + threadIdx.x, ray = ray0 + i_ray;
+    if (i_ray >= n_rays) return;
     const Ray r = make_ray(F, ray % F.W, ray / F.W);
     float beta[D];
 #pragma unroll
@@ -120,7 +144,7 @@ __global__ void composite_kernel(const FrameDesc F, const RenderConst rc, const 
     float T = 1.0f, C[3] = {0.0f, 0.0f, 0.0f};
     long long S = 0;
     int n_look = 0, n_occ = 0, n_steps = rc.N;
-    long long j = offset[ray];
+    long long j = offset[i_ray];
     float p[3];
     for (int i = 0; i < rc.N; ++i) {
         if (!sample_at(r, rc, b, i, p)) continue;
@@ -162,22 +186,21 @@ __global__ void composite_kernel(const FrameDesc F, const RenderConst rc, const 
 }
 
 template <int D>
-cudaError_t launch_composite(const FrameDesc &F, const RenderConst &rc, const Box &b, const float *pos_out,
-                             const float *dir_out, const long long *offset, cudaStream_t s) {
-    const int n = F.W * F.H;
-    composite_kernel<D><<<(n + 127) / 128, 128, 0, s>>>(F, rc, b, pos_out, dir_out, offset);
+cudaError_t launch_composite(const FrameDesc &F, const RenderConst &rc, const Box &b, int ray0, int n,
+                             const float *pos_out, const float *dir_out, const long long *offset, cudaStream_t s) {
+    composite_kernel<D><<<(n + 127) / 128, 128, 0, s>>>(F, rc, b, ray0, n, pos_out, dir_out, offset);
     return cudaGetLastError();
 }
 
-cudaError_t composite(int D, const FrameDesc &F, const RenderConst &rc, const Box &b, const float *pos_out,
-                      const float *dir_out, const long long *offset, cudaStream_t s) {
+cudaError_t composite(int D, const FrameDesc &F, const RenderConst &rc, const Box &b, int ray0, int n,
+                      const float *pos_out, const float *dir_out, const long long *offset, cudaStream_t s) {
     switch (D) {
-        case 1: return launch_composite<1>(F, rc, b, pos_out, dir_out, offset, s);
-        case 2: return launch_composite<2>(F, rc, b, pos_out, dir_out, offset, s);
-        case 4: return launch_composite<4>(F, rc, b, pos_out, dir_out, offset, s);
-        case 6: return launch_composite<6>(F, rc, b, pos_out, dir_out, offset, s);
-        case 8: return launch_composite<8>(F, rc, b, pos_out, dir_out, offset, s);
-        case 16: return launch_composite<16>(F, rc, b, pos_out, dir_out, offset, s);
+        case 1: return launch_composite<1>(F, rc, b, ray0, n, pos_out, dir_out, offset, s);
+        case 2: return launch_composite<2>(F, rc, b, ray0, n, pos_out, dir_out, offset, s);
+        case 4: return launch_composite<4>(F, rc, b, ray0, n, pos_out, dir_out, offset, s);
+        case 6: return launch_composite<6>(F, rc, b, ray0, n, pos_out, dir_out, offset, s);
+        case 8: return launch_composite<8>(F, rc, b, ray0, n, pos_out, dir_out, offset, s);
+        case 16: return launch_composite<16>(F, rc, b, ray0, n, pos_out, dir_out, offset, s);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -225,47 +248,56 @@ extern "C" fnr_status fnr_render_mlp(fnr_context *ctx, const fnr_mlp *pos_mlp, c
     FrameDesc F;
     fill_frame(&F, cam, rgba_dev, stats_dev, nullptr, 0);
     const long long n_rays = static_cast<long long>(cam->width) * cam->height;
-    // temporaries: the sample list is sized for every sample (the worst case), the rest per ray
+    // The budget is charged for temporaries of all samples at once; those of one batch are allocated, sized for
+    // every one of its samples.
     const long long max_pts = n_rays * rc.N;
     const uint64_t bytes = uint64_t(max_pts) * (3 + 1 + 3 * D) * 4 + uint64_t(n_rays) * (8 + 4 + 12 + 4 * D) + 8;
     if (!budget_charge(ctx, bytes))
         return fail(FNR_ERR_BUDGET, "the uncached render needs %llu bytes of temporaries",
                     (unsigned long long)bytes);
-    DevMem points, pos_out, dirs, dir_out, offset, count, total;
-    st = FNR_OK;
-    if ((e = dev_malloc(&points.p, size_t(max_pts) * 12)) != cudaSuccess ||
-        (e = dev_malloc(&pos_out.p, size_t(max_pts) * (1 + 3 * D) * 4)) != cudaSuccess ||
+    constexpr long long kBatchPoints = 1LL << 23;
+    const long long batch = std::min<long long>(n_rays, std::max<long long>(kBatchPoints / rc.N, 1));
+    const long long n_batches = (n_rays + batch - 1) / batch, batch_pts = batch * rc.N;
+    DevMem points, pos_out, dirs, dir_out, offset, totals;
+    PointsMlp pos, dir;
+    if ((e = dev_malloc(&points.p, size_t(batch_pts) * 12)) != cudaSuccess ||
+        (e = dev_malloc(&pos_out.p, size_t(batch_pts) * (1 + 3 * D) * 4)) != cudaSuccess ||
         (e = dev_malloc(&dirs.p, size_t(n_rays) * 12)) != cudaSuccess ||
         (e = dev_malloc(&dir_out.p, size_t(n_rays) * D * 4)) != cudaSuccess ||
-        (e = dev_malloc(&offset.p, size_t(n_rays) * 8)) != cudaSuccess ||
-        (e = dev_malloc(&count.p, size_t(n_rays) * 4)) != cudaSuccess ||
-        (e = dev_malloc(&total.p, 8)) != cudaSuccess)
+        (e = dev_malloc(&offset.p, size_t(batch) * 8)) != cudaSuccess ||
+        (e = dev_malloc(&totals.p, size_t(n_batches) * 8)) != cudaSuccess)
         st = cuda_fail(e, "uncached render temporaries");
-    unsigned long long n_pts = 0;
+    if (st == FNR_OK && (e = cudaMemsetAsync(totals.p, 0, size_t(n_batches) * 8, s)) != cudaSuccess)
+        st = cuda_fail(e, "memset");
+    if (st == FNR_OK) st = pos.prepare(pos_mlp, 1 + 3 * D, true, s);
+    if (st == FNR_OK) st = dir.prepare(dir_mlp, D, false, s);
     if (st == FNR_OK) {
-        if ((e = cudaMemsetAsync(total.p, 0, 8, s)) != cudaSuccess) st = cuda_fail(e, "memset");
+        directions_kernel<<<unsigned((n_rays + 127) / 128), 128, 0, s>>>(F, static_cast<float *>(dirs.p));
+        if ((e = cudaGetLastError()) != cudaSuccess) st = cuda_fail(e, "ray directions");
     }
-    if (st == FNR_OK) {
-        samples_kernel<<<unsigned((n_rays + 127) / 128), 128, 0, s>>>(
-            F, rc, b, static_cast<float *>(points.p), static_cast<unsigned long long *>(total.p),
-            static_cast<long long *>(offset.p), static_cast<int *>(count.p), static_cast<float *>(dirs.p));
-        if ((e = cudaGetLastError()) != cudaSuccess ||
-            (e = cudaMemcpyAsync(&n_pts, total.p, 8, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-            (e = cudaStreamSynchronize(s)) != cudaSuccess)
+    if (st == FNR_OK)
+        st = dir.launch(static_cast<const float *>(dirs.p), n_rays, nullptr, static_cast<float *>(dir_out.p),
+                        ctx->num_sms, s);
+    for (long long i = 0; i < n_batches && st == FNR_OK; ++i) {
+        const int ray0 = int(i * batch), n = int(std::min(batch, n_rays - i * batch));
+        unsigned long long *total = static_cast<unsigned long long *>(totals.p) + i;
+        samples_kernel<<<unsigned((n + 127) / 128), 128, 0, s>>>(F, rc, b, ray0, n, static_cast<float *>(points.p), total,
+                                                                 static_cast<long long *>(offset.p));
+        if ((e = cudaGetLastError()) != cudaSuccess) {
             st = cuda_fail(e, "sample positions");
-    }
-    if (st == FNR_OK)
-        st = run_mlp_points(pos_mlp, static_cast<const float *>(points.p), (long long)n_pts,
-                            static_cast<float *>(pos_out.p), 1 + 3 * D, true, ctx->num_sms, s);
-    if (st == FNR_OK)
-        st = run_mlp_points(dir_mlp, static_cast<const float *>(dirs.p), n_rays, static_cast<float *>(dir_out.p), D,
-                            false, ctx->num_sms, s);
-    if (st == FNR_OK) {
-        if ((e = composite(D, F, rc, b, static_cast<const float *>(pos_out.p), static_cast<const float *>(dir_out.p),
-                           static_cast<const long long *>(offset.p), s)) != cudaSuccess ||
-            (e = cudaStreamSynchronize(s)) != cudaSuccess)
+            break;
+        }
+        st = pos.launch(static_cast<const float *>(points.p), (long long)n * rc.N, total,
+                        static_cast<float *>(pos_out.p), ctx->num_sms, s);
+        if (st == FNR_OK &&
+            (e = composite(D, F, rc, b, ray0, n, static_cast<const float *>(pos_out.p),
+                           static_cast<const float *>(dir_out.p), static_cast<const long long *>(offset.p), s)) !=
+                cudaSuccess)
             st = cuda_fail(e, "uncached composite");
     }
+    if (st == FNR_OK) st = pos.finish(s);
+    if (st == FNR_OK) st = dir.finish(s);
+    if (st != FNR_OK) cudaStreamSynchronize(s);  // whatever was launched has left the temporaries
     budget_uncharge(ctx, bytes);
     return st;
 }
