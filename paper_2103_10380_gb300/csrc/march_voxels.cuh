@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(FNR_BLOCK) march_voxels_kernel(const __grid_co
     // bricks in one step (VoxelWalk::pass_cube), from the cache's distance field.
     const bool jumps = FORM == kVoxJump && skip && F.cells == nullptr && c.dist != nullptr;
     float T = 1.0f, Cr = 0.0f, Cg = 0.0f, Cb = 0.0f;
-    long long S = 0;
+    unsigned long long S = 0;
     int n_gen = 0, n_steps = 0, n_look = 0, n_occ = 0;
     bool term = false;
     const long long pix = active ? static_cast<long long>(py) * F.W + px : 0;
@@ -326,9 +326,8 @@ __global__ void __launch_bounds__(FNR_BLOCK) march_voxels_kernel(const __grid_co
                 wgt[u] = T * alpha;
                 T = T * ext;
                 occ |= 1u << u;
-                const long long qd = fixed_depth(od);
-                S = (S > 0x7fffffffffffffffLL - qd) ? 0x7fffffffffffffffLL : S + qd;
-                if (S >= r.s_thr) term = true;
+                if (od > 0.0f) S += fixed_depth(od);
+                if (S >= static_cast<unsigned long long>(r.s_thr)) term = true;
             }
         }
         // records of the composited cells, colour added in walk order

@@ -142,7 +142,7 @@ __global__ void composite_kernel(const FrameDesc F, const RenderConst rc, const 
 #pragma unroll
     for (int i = 0; i < D; ++i) beta[i] = dir_out[static_cast<long long>(ray) * D + i];
     float T = 1.0f, C[3] = {0.0f, 0.0f, 0.0f};
-    long long S = 0;
+    unsigned long long S = 0;
     int n_look = 0, n_occ = 0, n_steps = rc.N;
     long long j = offset[i_ray];
     float p[3];
@@ -169,9 +169,8 @@ __global__ void composite_kernel(const FrameDesc F, const RenderConst rc, const 
         C[1] = __fmaf_rn(w, col[1], C[1]);
         C[2] = __fmaf_rn(w, col[2], C[2]);
         T = T * ext;
-        const long long qd = dev::fixed_depth(sg);
-        S = (S > 0x7fffffffffffffffLL - qd) ? 0x7fffffffffffffffLL : S + qd;
-        if (S >= rc.s_thr) {
+        S += dev::fixed_depth(sg);
+        if (S >= static_cast<unsigned long long>(rc.s_thr)) {
             n_steps = i + 1;
             break;
         }
