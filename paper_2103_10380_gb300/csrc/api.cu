@@ -176,14 +176,6 @@ bool budget_charge(fnr_context *ctx, uint64_t bytes) {
 
 void budget_uncharge(fnr_context *ctx, uint64_t bytes) { ctx->used.fetch_sub(bytes); }
 
-// RAII device buffer for build-time temporaries.
-struct DevBuf {
-    void *p = nullptr;
-    ~DevBuf() {
-        if (p) cudaFree(p);
-    }
-};
-
 static fnr_status build_from_arrays(fnr_cache *c, const fnr_cache_source *src, const Layout &L, bool records,
                                     cudaStream_t s) {
     const fnr_cache_desc &d = c->desc;
@@ -197,9 +189,9 @@ static fnr_status build_from_arrays(fnr_cache *c, const fnr_cache_source *src, c
     // Slab size for staging host arrays (cells per slab, whole x-rows).
     const int64_t fit = (int64_t(256) << 20) / (4 * (nch + 1)) / d.k * d.k;
     const int64_t slab = dev ? k3 : std::max<int64_t>(d.k, std::min<int64_t>(k3, fit));
-    DevBuf stage;
+    TempBuf stage;
     if (!dev) {
-        if ((e = dev_malloc(&stage.p, size_t(slab) * 4 * (nch + 1))) != cudaSuccess) return cuda_fail(e, "staging");
+        if ((e = stage.alloc(c->ctx, size_t(slab) * 4 * (nch + 1), s)) != cudaSuccess) return cuda_fail(e, "staging");
     }
     auto slab_ptrs = [&](int64_t c0, int64_t n, const float **sp, const float **up) -> cudaError_t {
         if (dev) {
@@ -222,9 +214,9 @@ static fnr_status build_from_arrays(fnr_cache *c, const fnr_cache_source *src, c
         // (1) per offset brick and channel the min and max, and the absmax of the density; (2) the binary16
         // midranges and, from the same extremes, the absmax of the residuals; (3) the scales
         const int64_t nbo3 = int64_t(odim) * odim * odim;
-        DevBuf amax, kmm;
-        if ((e = dev_malloc(&amax.p, sizeof(unsigned) * (1 + nch))) != cudaSuccess) return cuda_fail(e, "absmax");
-        if ((e = dev_malloc(&kmm.p, sizeof(unsigned) * 2 * size_t(nbo3) * nch)) != cudaSuccess)
+        TempBuf amax, kmm;
+        if ((e = amax.alloc(c->ctx, sizeof(unsigned) * (1 + nch), s)) != cudaSuccess) return cuda_fail(e, "absmax");
+        if ((e = kmm.alloc(c->ctx, sizeof(unsigned) * 2 * size_t(nbo3) * nch, s)) != cudaSuccess)
             return cuda_fail(e, "offset min / max");
         unsigned *kmin = static_cast<unsigned *>(kmm.p), *kmax = kmin + size_t(nbo3) * nch;
         unsigned *amx = static_cast<unsigned *>(amax.p);
@@ -246,7 +238,6 @@ static fnr_status build_from_arrays(fnr_cache *c, const fnr_cache_source *src, c
             return cuda_fail(e, "offsets kernel");
         if ((e = launch_scales_from_absmax(amx, scales, 1 + nch, s)) != cudaSuccess)
             return cuda_fail(e, "scales kernel");
-        if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "scales sync");
     }
     for (int64_t c0 = 0; c0 < k3; c0 += slab) {
         const int64_t n = std::min(slab, k3 - c0);
@@ -264,16 +255,16 @@ static fnr_status build_from_arrays(fnr_cache *c, const fnr_cache_source *src, c
     // direction cache
     const int64_t nb = int64_t(d.l) * d.l * d.D;
     const float *bp = src->beta;
-    DevBuf bstage;
+    TempBuf bstage;
     if (!dev) {
-        if ((e = dev_malloc(&bstage.p, size_t(nb) * 4)) != cudaSuccess) return cuda_fail(e, "beta staging");
+        if ((e = bstage.alloc(c->ctx, size_t(nb) * 4, s)) != cudaSuccess) return cuda_fail(e, "beta staging");
         if ((e = cudaMemcpyAsync(bstage.p, src->beta, size_t(nb) * 4, cudaMemcpyHostToDevice, s)) != cudaSuccess)
             return cuda_fail(e, "beta upload");
         bp = static_cast<const float *>(bstage.p);
     }
     if ((e = launch_convert_beta(bp, base + L.off_beta, nb, d.dir_precision, s)) != cudaSuccess)
         return cuda_fail(e, "beta conversion");
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "build sync");
+    if (!dev && (e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "build sync");
     return FNR_OK;
 }
 
@@ -407,6 +398,17 @@ fnr_status fnr_context_create(int32_t device, uint64_t hbm_budget_bytes, fnr_con
     ctx->device = device;
     ctx->budget = hbm_budget_bytes;
     cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device);
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    uint64_t keep = kPoolKeepBytes;
+    if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess) {
+        ctx->pool = nullptr;
+        cudaGetLastError();
+    } else if (cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+    }
     *out = ctx;
     return FNR_OK;
 }
@@ -427,6 +429,10 @@ fnr_status fnr_context_destroy(fnr_context *ctx) {
     for (fnr_cache *c : cs) {
         if (c->owned && c->base) cudaFree(c->base);
         delete c;
+    }
+    if (ctx->pool) {
+        cudaDeviceSynchronize();  // temporaries are freed in stream order
+        cudaMemPoolDestroy(ctx->pool);
     }
     delete ctx;
     return FNR_OK;
@@ -455,7 +461,7 @@ uint64_t fnr_cache_footprint(const fnr_cache_desc *d) {
 }
 
 static fnr_status build_dense(fnr_context *ctx, const fnr_cache_desc *desc, const fnr_cache_source *src,
-                              bool records, cudaStream_t s, fnr_cache **out);
+                              bool records, TempBuf *stage, cudaStream_t s, fnr_cache **out);
 
 // Dense cache -> FNR_LAYOUT_BRICKS cache: pool slots in brick-index order of
 // the occupied bricks, found on the GPU (only their count is read back, for the
@@ -467,9 +473,9 @@ static fnr_status make_bricks(fnr_context *ctx, const fnr_cache *dense, const La
     const CacheView &dv = dense->view;
     const int64_t nb = dv.occ_dim, nb3 = nb * nb * nb, n_words = int64_t(occupancy_words(desc));
     cudaError_t e;
-    DevBuf rank;
+    TempBuf rank;
     uint32_t total = 0;
-    if ((e = dev_malloc(&rank.p, size_t(n_words + 1) * 4)) != cudaSuccess) return cuda_fail(e, "brick ranks");
+    if ((e = rank.alloc(ctx, size_t(n_words + 1) * 4, s)) != cudaSuccess) return cuda_fail(e, "brick ranks");
     uint32_t *rk = static_cast<uint32_t *>(rank.p);
     if ((e = launch_brick_rank(dv.occ, n_words, rk, rk + n_words, s)) != cudaSuccess ||
         (e = cudaMemcpyAsync(&total, rk + n_words, 4, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
@@ -493,9 +499,9 @@ static fnr_status make_bricks(fnr_context *ctx, const fnr_cache *dense, const La
     }
     char *base = static_cast<char *>(c->base);
     const char *dbase = static_cast<const char *>(dense->base);
-    DevBuf slots;
+    TempBuf slots;
     fnr_status st = FNR_OK;
-    if ((e = dev_malloc(&slots.p, size_t(std::max<int64_t>(n_bricks, 1)) * 4)) != cudaSuccess) st = cuda_fail(e, "slots");
+    if ((e = slots.alloc(ctx, size_t(std::max<int64_t>(n_bricks, 1)) * 4, s)) != cudaSuccess) st = cuda_fail(e, "slots");
     const int32_t *sb = static_cast<const int32_t *>(slots.p);
     if (st == FNR_OK &&
         ((e = launch_brick_pages(dv.occ, rk, nb3, reinterpret_cast<int32_t *>(base + L.off_page),
@@ -549,19 +555,22 @@ fnr_status fnr_build_cache(fnr_context *ctx, const fnr_cache_desc *desc, const f
         dd.layout = FNR_LAYOUT_DENSE;
         const bool direct = src->kind == FNR_SRC_ARRAYS && src->location == FNR_LOC_DEVICE;
         fnr_cache *dense = nullptr;
-        fnr_status st = build_dense(ctx, &dd, src, !direct, s, &dense);
+        TempBuf stage;
+        fnr_status st = build_dense(ctx, &dd, src, !direct, &stage, s, &dense);
         if (st != FNR_OK) return st;
         st = make_bricks(ctx, dense, layout_of(&dd, -1, !direct), direct ? src->uvw : nullptr, desc, s, out);
-        std::string msg = st != FNR_OK ? std::string(fnr_last_error()) : std::string();
-        fnr_cache_free(ctx, dense);
-        if (st != FNR_OK) return fail(st, "%s", msg.c_str());
-        return FNR_OK;
+        budget_uncharge(ctx, dense->footprint);
+        delete dense;
+        return st;
     }
-    return build_dense(ctx, desc, src, true, s, out);
+    return build_dense(ctx, desc, src, true, nullptr, s, out);
 }
 
+
+// A dense cache, complete on return; or, with `stage`, the dense stage of a brick build in that buffer, complete in
+// the order of the stream (the caller deletes it and returns its charge, c->footprint).
 static fnr_status build_dense(fnr_context *ctx, const fnr_cache_desc *desc, const fnr_cache_source *src,
-                              bool records, cudaStream_t s, fnr_cache **out) {
+                              bool records, TempBuf *stage, cudaStream_t s, fnr_cache **out) {
     fnr_status st0;
     if (src->kind == FNR_SRC_MLP) {
         if ((st0 = check_mlp(src->pos_mlp, 1 + 3 * desc->D, "pos_mlp")) != FNR_OK) return st0;
@@ -575,7 +584,7 @@ static fnr_status build_dense(fnr_context *ctx, const fnr_cache_desc *desc, cons
     } else {
         return fail(FNR_ERR_INVALID_ARG, "unknown source kind %d", src->kind);
     }
-    cudaError_t e = cudaSetDevice(ctx->device);
+    cudaError_t e = use_device(ctx->device);
     if (e != cudaSuccess) return cuda_fail(e, "cudaSetDevice");
     const Layout L = layout_of(desc, -1, records);
     const uint64_t charge = layout_of(desc).total;
@@ -586,34 +595,41 @@ static fnr_status build_dense(fnr_context *ctx, const fnr_cache_desc *desc, cons
     c->desc = *desc;
     c->footprint = charge;
     c->ctx = ctx;
-    if ((e = dev_malloc(&c->base, L.total)) != cudaSuccess) {
+    if (stage) {
+        e = stage->alloc(ctx, L.total, s);
+        c->base = stage->p;
+        c->owned = false;
+    } else {
+        e = dev_malloc(&c->base, L.total);
+    }
+    if (e != cudaSuccess) {
         budget_uncharge(ctx, charge);
         delete c;
         return cuda_fail(e, "cache allocation");
     }
+    // The direction-bin tables and, where no build computes them, defined scales (1): adjacent sections, one upload
+    // (from pageable memory: the call returns when the buffer has been read).
     std::vector<float> ct, qp;
     bin_tables(desc->l, ct, qp);
+    const bool fp8 = desc->pos_precision == FNR_PREC_FP8_E4M3;
+    const size_t n_ones = fp8 ? 0 : size_t(1 + 3 * desc->D);
+    std::vector<char> tables(size_t(L.off_scales - L.off_ct) + n_ones * 4, 0);
+    memcpy(tables.data(), ct.data(), ct.size() * 4);
+    memcpy(tables.data() + (L.off_qp - L.off_ct), qp.data(), qp.size() * 4);
+    const std::vector<float> ones(n_ones, 1.0f);
+    if (n_ones) memcpy(tables.data() + (L.off_scales - L.off_ct), ones.data(), n_ones * 4);
     char *base = static_cast<char *>(c->base);
     fnr_status st = FNR_OK;
-    if ((e = cudaMemcpyAsync(base + L.off_ct, ct.data(), ct.size() * 4, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(base + L.off_qp, qp.data(), qp.size() * 4, cudaMemcpyHostToDevice, s)) != cudaSuccess) {
+    if ((e = cudaMemcpyAsync(base + L.off_ct, tables.data(), tables.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess)
         st = cuda_fail(e, "table upload");
-    }
-    if (st == FNR_OK && desc->pos_precision != FNR_PREC_FP8_E4M3) {
-        // scales unused: keep them defined (1.0)
-        std::vector<float> ones(1 + 3 * desc->D, 1.0f);
-        if ((e = cudaMemcpyAsync(base + L.off_scales, ones.data(), ones.size() * 4, cudaMemcpyHostToDevice, s)) !=
-            cudaSuccess)
-            st = cuda_fail(e, "scale upload");
-        if (st == FNR_OK && (e = cudaStreamSynchronize(s)) != cudaSuccess) st = cuda_fail(e, "sync");
-    }
+    GridMlp pos, dir;
     if (st == FNR_OK) {
         if (src->kind == FNR_SRC_ARRAYS) {
             st = build_from_arrays(c, src, L, records, s);
         } else {
             fill_view(c, L);
-            st = run_mlp(src->pos_mlp, 0, c->desc, c->view, ctx->num_sms, s);
-            if (st == FNR_OK) st = run_mlp(src->dir_mlp, 1, c->desc, c->view, ctx->num_sms, s);
+            st = pos.launch(ctx, src->pos_mlp, 0, c->desc, c->view, s);
+            if (st == FNR_OK) st = dir.launch(ctx, src->dir_mlp, 1, c->desc, c->view, s);
         }
     }
     if (st == FNR_OK) {
@@ -623,18 +639,23 @@ static fnr_status build_dense(fnr_context *ctx, const fnr_cache_desc *desc, cons
             (e = launch_occupancy(c->view, reinterpret_cast<uint32_t *>(base + L.off_occ), s)) != cudaSuccess ||
             (e = launch_brick_distance(reinterpret_cast<const uint32_t *>(base + L.off_occ), c->view.occ_dim,
                                        c->view.occ_shift, reinterpret_cast<uint8_t *>(base + L.off_dist),
-                                       c->view.dist_dim, c->view.dist_shift, s)) != cudaSuccess ||
-            (e = cudaStreamSynchronize(s)) != cudaSuccess)
+                                       c->view.dist_dim, c->view.dist_shift, s)) != cudaSuccess)
             st = cuda_fail(e, "occupancy bits");
     }
+    // one wait for everything queued (a stage's is that for the number of its bricks)
+    if (st == FNR_OK && src->kind == FNR_SRC_MLP) {
+        st = pos.finish(s);
+        if (st == FNR_OK) st = dir.finish(s);
+    } else if (st == FNR_OK && !stage && (e = cudaStreamSynchronize(s)) != cudaSuccess) {
+        st = cuda_fail(e, "build sync");
+    }
     if (st != FNR_OK) {
-        cudaFree(c->base);
+        if (c->owned) cudaFree(c->base);
         budget_uncharge(ctx, charge);
         delete c;
         return st;
     }
-    fill_view(c, L);
-    {
+    if (!stage) {
         std::lock_guard<std::mutex> g(ctx->mu);
         ctx->caches.insert(c);
     }
@@ -737,7 +758,7 @@ fnr_status fnr_cache_load(fnr_context *ctx, const char *path, fnr_stream_t strea
     if (h.footprint != L.total)
         return fail(FNR_ERR_IO, "%s: footprint %llu does not match the descriptor's %llu", path,
                     (unsigned long long)h.footprint, (unsigned long long)L.total);
-    cudaError_t e = cudaSetDevice(ctx->device);
+    cudaError_t e = use_device(ctx->device);
     if (e != cudaSuccess) return cuda_fail(e, "cudaSetDevice");
     if (!budget_charge(ctx, L.total))
         return fail(FNR_ERR_BUDGET, "cache needs %llu bytes, budget %llu, in use %llu", (unsigned long long)L.total,
@@ -826,7 +847,7 @@ fnr_status fnr_render(fnr_context *ctx, const fnr_cache *cache, const fnr_camera
         return fail(FNR_ERR_UNSUPPORTED, "the voxel walk reads dense caches only");
     for (int i = 0; i < n_cams; ++i)
         if ((st = check_camera(&cams[i])) != FNR_OK) return st;
-    cudaError_t e = cudaSetDevice(ctx->device);
+    cudaError_t e = use_device(ctx->device);
     if (e != cudaSuccess) return cuda_fail(e, "cudaSetDevice");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     MarchArgs a;

@@ -108,6 +108,31 @@ template <class T>
 cudaError_t dev_malloc(T **p, size_t bytes) {
     return dev_malloc(reinterpret_cast<void **>(p), bytes);
 }
+// A temporary of one call, freed with the object in the order of stream `s`. Up to kPooledBytes it comes from the
+// context's pool of stream-ordered memory (a cudaMalloc and cudaFree pair takes 60 us, a small build had seven);
+// larger ones are allocated and freed (from a pool that does not keep them they cost twice as much). The pool
+// belongs to one context, keeps at most kPoolKeepBytes between calls and is given back with the context; streams
+// and threads may share it.
+constexpr size_t kPooledBytes = size_t(64) << 20, kPoolKeepBytes = size_t(128) << 20;
+class TempBuf {
+public:
+    void *p = nullptr;
+    TempBuf() = default;
+    TempBuf(const TempBuf &) = delete;
+    TempBuf &operator=(const TempBuf &) = delete;
+    ~TempBuf() { release(); }
+    cudaError_t alloc(const fnr_context *ctx, size_t bytes, cudaStream_t s);
+    void release();
+
+private:
+    bool pooled = false;
+    cudaStream_t stream = nullptr;
+};
+// Make the device current, if it is not.
+inline cudaError_t use_device(int device) {
+    int cur = -1;
+    return cudaGetDevice(&cur) == cudaSuccess && cur == device ? cudaSuccess : cudaSetDevice(device);
+}
 // The armed cache-build fault (fnr_testing_mlp_fault), taken once: leaves the
 // arguments unchanged when none is armed.
 void take_mlp_fault(long long *wait_limit, long long *withhold);
@@ -172,11 +197,23 @@ fnr_status check_mlp(const fnr_mlp *m, int n_out_min, const char *name);
 // The same at listed points: prepare() lays the weights out once, each launch() evaluates [n][3] points on the
 // device (n read from n_dev, at most max_n; n = max_n if n_dev is null), the first out_stride head outputs of
 // point p going to out[p * out_stride + c] in FP32 (channel 0 through ReLU if relu0), finish() waits and reports.
+// GridMlp is F over a cache's grid (mode 0: F_pos over the cells, 1: F_dir over the bins): launch() queues the
+// evaluation, finish() waits and reports.
 class PointsMlp {
 public:
     ~PointsMlp();
-    fnr_status prepare(const fnr_mlp *m, int out_stride, bool relu0, cudaStream_t s);
-    fnr_status launch(const float *points, long long max_n, const unsigned long long *n_dev, float *out, int num_sms,
+    fnr_status prepare(const fnr_context *ctx, const fnr_mlp *m, int out_stride, bool relu0, cudaStream_t s);
+    fnr_status launch(const float *points, long long max_n, const unsigned long long *n_dev, float *out, cudaStream_t s);
+    fnr_status finish(cudaStream_t s);
+
+private:
+    struct Impl;
+    Impl *impl = nullptr;
+};
+class GridMlp {
+public:
+    ~GridMlp();
+    fnr_status launch(const fnr_context *ctx, const fnr_mlp *m, int mode, const fnr_cache_desc &d, const CacheView &v,
                       cudaStream_t s);
     fnr_status finish(cudaStream_t s);
 
@@ -184,8 +221,6 @@ private:
     struct Impl;
     Impl *impl = nullptr;
 };
-fnr_status run_mlp(const fnr_mlp *m, int mode, const fnr_cache_desc &d, const CacheView &v, int num_sms,
-                   cudaStream_t s);
 
 }  // namespace fnr
 
@@ -209,4 +244,5 @@ struct fnr_context {
     std::set<fnr_cache *> caches;
     std::mutex serve_mu;
     fnr::Server *server = nullptr;
+    cudaMemPool_t pool = nullptr;  // temporaries (TempBuf); null if the device has no such pools
 };

@@ -626,26 +626,23 @@ namespace {
 
 // Device copies of one network's weights and biases, and the error word of its launches.
 struct MlpBuffers {
-    void *weights = nullptr, *biases = nullptr, *err = nullptr;
-    ~MlpBuffers() {
-        if (weights) cudaFree(weights);
-        if (biases) cudaFree(biases);
-        if (err) cudaFree(err);
-    }
+    TempBuf weights, biases, err;
+    int num_sms = 0;
 };
 
 // Lay out the weights and biases of m and fill the layer table of A (A.mode and its outputs per point are set).
-fnr_status mlp_prepare(const fnr_mlp *m, MlpArgs &A, MlpBuffers &B, cudaStream_t s) {
+fnr_status mlp_prepare(const fnr_context *ctx, const fnr_mlp *m, MlpArgs &A, MlpBuffers &B, cudaStream_t s) {
+    B.num_sms = ctx->num_sms;
     size_t welems = 0, belems = 0;
     for (int i = 0; i < m->n_layers; ++i) {
         welems += size_t(round16(m->dims[i + 1])) * round64(m->dims[i]);
         belems += size_t(round16(m->dims[i + 1]));
     }
     cudaError_t e;
-    if ((e = dev_malloc(&B.weights, welems * 2)) != cudaSuccess) return cuda_fail(e, "MLP weights");
-    if ((e = dev_malloc(&B.biases, belems * 4)) != cudaSuccess) return cuda_fail(e, "MLP biases");
-    if ((e = dev_malloc(&B.err, 4)) != cudaSuccess) return cuda_fail(e, "MLP error word");
-    if ((e = cudaMemsetAsync(B.err, 0, 4, s)) != cudaSuccess) return cuda_fail(e, "memset");
+    if ((e = B.weights.alloc(ctx, welems * 2, s)) != cudaSuccess) return cuda_fail(e, "MLP weights");
+    if ((e = B.biases.alloc(ctx, belems * 4, s)) != cudaSuccess) return cuda_fail(e, "MLP biases");
+    if ((e = B.err.alloc(ctx, 4, s)) != cudaSuccess) return cuda_fail(e, "MLP error word");
+    if ((e = cudaMemsetAsync(B.err.p, 0, 4, s)) != cudaSuccess) return cuda_fail(e, "memset");
     A.n_out = A.mode == 0 ? 1 + 3 * A.D : (A.mode == 1 ? A.D : A.out_stride);
     if (A.n_out < 1 || A.n_out > kMaxOut || A.n_out > m->dims[m->n_layers])
         return fail(FNR_ERR_UNSUPPORTED, "MLP kernel: %d outputs per point (at most %d)", A.n_out, kMaxOut);
@@ -656,11 +653,11 @@ fnr_status mlp_prepare(const fnr_mlp *m, MlpArgs &A, MlpBuffers &B, cudaStream_t
     for (int i = 0; i < m->n_layers; ++i) {
         // the head is evaluated up to the outputs that are stored
         const int K = m->dims[i], N = i + 1 == m->n_layers ? A.n_out : m->dims[i + 1], Kp = round64(K), Np = round16(N);
-        uint16_t *wd = static_cast<uint16_t *>(B.weights) + wo;
+        uint16_t *wd = static_cast<uint16_t *>(B.weights.p) + wo;
         P.w[i] = m->weights[i];
         P.b[i] = m->biases[i];
         P.w_out[i] = wd;
-        P.b_out[i] = static_cast<float *>(B.biases) + bo;
+        P.b_out[i] = static_cast<float *>(B.biases.p) + bo;
         P.N[i] = N;
         P.K[i] = K;
         P.Np[i] = Np;
@@ -675,11 +672,11 @@ fnr_status mlp_prepare(const fnr_mlp *m, MlpArgs &A, MlpBuffers &B, cudaStream_t
     }
     prepare_kernel<<<dim3(unsigned((max_elems + 255) / 256), unsigned(m->n_layers)), 256, 0, s>>>(P);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "MLP weight layout");
-    A.bias = static_cast<const float *>(B.biases);
+    A.bias = static_cast<const float *>(B.biases.p);
     A.n_bias = int(bo);
     A.n_layers = m->n_layers;
     A.pe_freqs = m->pe_freqs;
-    A.err = static_cast<int *>(B.err);
+    A.err = static_cast<int *>(B.err.p);
     A.wait_limit = kWaitLimit;
     A.withhold = -1;
     take_mlp_fault(&A.wait_limit, &A.withhold);
@@ -706,10 +703,17 @@ fnr_status mlp_finish(const MlpArgs &A, cudaStream_t s) {
 
 }  // namespace
 
-// Evaluate one MLP over its grid into the cache (mode 0: F_pos, 1: F_dir).
-fnr_status run_mlp(const fnr_mlp *m, int mode, const fnr_cache_desc &d, const CacheView &v, int num_sms,
-                   cudaStream_t s) {
+struct GridMlp::Impl {
     MlpArgs A;
+    MlpBuffers B;
+};
+
+GridMlp::~GridMlp() { delete impl; }
+
+fnr_status GridMlp::launch(const fnr_context *ctx, const fnr_mlp *m, int mode, const fnr_cache_desc &d,
+                           const CacheView &v, cudaStream_t s) {
+    impl = new Impl();
+    MlpArgs &A = impl->A;
     memset(&A, 0, sizeof(A));
     A.mode = mode;
     A.k = d.k;
@@ -726,11 +730,11 @@ fnr_status run_mlp(const fnr_mlp *m, int mode, const fnr_cache_desc &d, const Ca
     A.D = d.D;
     A.beta_out = const_cast<void *>(v.beta);
     A.dprec = d.dir_precision;
-    MlpBuffers B;
-    fnr_status st = mlp_prepare(m, A, B, s);
-    if (st == FNR_OK) st = mlp_launch(A, num_sms, s);
-    return st == FNR_OK ? mlp_finish(A, s) : st;
+    const fnr_status st = mlp_prepare(ctx, m, A, impl->B, s);
+    return st == FNR_OK ? mlp_launch(A, impl->B.num_sms, s) : st;
 }
+
+fnr_status GridMlp::finish(cudaStream_t s) { return mlp_finish(impl->A, s); }
 
 struct PointsMlp::Impl {
     MlpArgs A;
@@ -739,23 +743,23 @@ struct PointsMlp::Impl {
 
 PointsMlp::~PointsMlp() { delete impl; }
 
-fnr_status PointsMlp::prepare(const fnr_mlp *m, int out_stride, bool relu0, cudaStream_t s) {
+fnr_status PointsMlp::prepare(const fnr_context *ctx, const fnr_mlp *m, int out_stride, bool relu0, cudaStream_t s) {
     impl = new Impl();
     memset(&impl->A, 0, sizeof(impl->A));
     impl->A.mode = 2;
     impl->A.out_stride = out_stride;
     impl->A.relu0 = relu0 ? 1 : 0;
-    return mlp_prepare(m, impl->A, impl->B, s);
+    return mlp_prepare(ctx, m, impl->A, impl->B, s);
 }
 
 fnr_status PointsMlp::launch(const float *points, long long max_n, const unsigned long long *n_dev, float *out,
-                             int num_sms, cudaStream_t s) {
+                             cudaStream_t s) {
     MlpArgs A = impl->A;
     A.n_points = max_n;
     A.n_dev = n_dev;
     A.points = points;
     A.out = out;
-    return mlp_launch(A, num_sms, s);
+    return mlp_launch(A, impl->B.num_sms, s);
 }
 
 fnr_status PointsMlp::finish(cudaStream_t s) { return mlp_finish(impl->A, s); }

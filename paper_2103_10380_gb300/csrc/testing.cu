@@ -1,5 +1,5 @@
 // testing.cu -- test hooks (fnr_testing.h): failure injection and the choice
-// of the cache-build kernel's form; and the one device allocation helper every
+// of the cache-build kernel's form; and the device allocation helpers every
 // library allocation goes through.
 #include <atomic>
 
@@ -19,17 +19,37 @@ std::atomic<int> g_mlp_cta_pair{0};
 
 bool mlp_cta_pair() { return g_mlp_cta_pair.load() != 0; }
 
-cudaError_t dev_malloc(void **p, size_t bytes) {
-    if (g_alloc_fail.load() > 0) {
-        if (g_alloc_skip.load() > 0) {
-            g_alloc_skip.fetch_sub(1);
-        } else {
-            g_alloc_fail.fetch_sub(1);
-            *p = nullptr;
-            return cudaErrorMemoryAllocation;
-        }
+// Whether the next allocation is one of those made to fail.
+static bool injected_failure() {
+    if (g_alloc_fail.load() <= 0) return false;
+    if (g_alloc_skip.load() > 0) {
+        g_alloc_skip.fetch_sub(1);
+        return false;
     }
-    return cudaMalloc(p, bytes);
+    g_alloc_fail.fetch_sub(1);
+    return true;
+}
+
+cudaError_t dev_malloc(void **p, size_t bytes) {
+    *p = nullptr;
+    return injected_failure() ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+}
+
+cudaError_t TempBuf::alloc(const fnr_context *ctx, size_t bytes, cudaStream_t s) {
+    release();
+    if (injected_failure()) return cudaErrorMemoryAllocation;
+    pooled = ctx->pool && bytes <= kPooledBytes;
+    stream = s;
+    const cudaError_t e = pooled ? cudaMallocFromPoolAsync(&p, bytes, ctx->pool, s) : cudaMalloc(&p, bytes);
+    if (e != cudaSuccess) p = nullptr;
+    return e;
+}
+
+void TempBuf::release() {
+    if (!p) return;
+    if (pooled) cudaFreeAsync(p, stream);
+    else cudaFree(p);
+    p = nullptr;
 }
 
 void take_mlp_fault(long long *wait_limit, long long *withhold) {

@@ -204,13 +204,6 @@ cudaError_t composite(int D, const FrameDesc &F, const RenderConst &rc, const Bo
     }
 }
 
-struct DevMem {
-    void *p = nullptr;
-    ~DevMem() {
-        if (p) cudaFree(p);
-    }
-};
-
 }  // namespace
 
 }  // namespace fnr
@@ -241,7 +234,7 @@ extern "C" fnr_status fnr_render_mlp(fnr_context *ctx, const fnr_mlp *pos_mlp, c
     if ((st = make_render_const(params, &rc)) != FNR_OK) return st;
     if (rc.flags != 0u) return fail(FNR_ERR_UNSUPPORTED, "the uncached render takes no render flags");
     if ((st = check_camera(cam)) != FNR_OK) return st;
-    cudaError_t e = cudaSetDevice(ctx->device);
+    cudaError_t e = use_device(ctx->device);
     if (e != cudaSuccess) return cuda_fail(e, "cudaSetDevice");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     FrameDesc F;
@@ -257,26 +250,25 @@ extern "C" fnr_status fnr_render_mlp(fnr_context *ctx, const fnr_mlp *pos_mlp, c
     constexpr long long kBatchPoints = 1LL << 23;
     const long long batch = std::min<long long>(n_rays, std::max<long long>(kBatchPoints / rc.N, 1));
     const long long n_batches = (n_rays + batch - 1) / batch, batch_pts = batch * rc.N;
-    DevMem points, pos_out, dirs, dir_out, offset, totals;
+    TempBuf points, pos_out, dirs, dir_out, offset, totals;
     PointsMlp pos, dir;
-    if ((e = dev_malloc(&points.p, size_t(batch_pts) * 12)) != cudaSuccess ||
-        (e = dev_malloc(&pos_out.p, size_t(batch_pts) * (1 + 3 * D) * 4)) != cudaSuccess ||
-        (e = dev_malloc(&dirs.p, size_t(n_rays) * 12)) != cudaSuccess ||
-        (e = dev_malloc(&dir_out.p, size_t(n_rays) * D * 4)) != cudaSuccess ||
-        (e = dev_malloc(&offset.p, size_t(batch) * 8)) != cudaSuccess ||
-        (e = dev_malloc(&totals.p, size_t(n_batches) * 8)) != cudaSuccess)
+    if ((e = points.alloc(ctx, size_t(batch_pts) * 12, s)) != cudaSuccess ||
+        (e = pos_out.alloc(ctx, size_t(batch_pts) * (1 + 3 * D) * 4, s)) != cudaSuccess ||
+        (e = dirs.alloc(ctx, size_t(n_rays) * 12, s)) != cudaSuccess ||
+        (e = dir_out.alloc(ctx, size_t(n_rays) * D * 4, s)) != cudaSuccess ||
+        (e = offset.alloc(ctx, size_t(batch) * 8, s)) != cudaSuccess ||
+        (e = totals.alloc(ctx, size_t(n_batches) * 8, s)) != cudaSuccess)
         st = cuda_fail(e, "uncached render temporaries");
     if (st == FNR_OK && (e = cudaMemsetAsync(totals.p, 0, size_t(n_batches) * 8, s)) != cudaSuccess)
         st = cuda_fail(e, "memset");
-    if (st == FNR_OK) st = pos.prepare(pos_mlp, 1 + 3 * D, true, s);
-    if (st == FNR_OK) st = dir.prepare(dir_mlp, D, false, s);
+    if (st == FNR_OK) st = pos.prepare(ctx, pos_mlp, 1 + 3 * D, true, s);
+    if (st == FNR_OK) st = dir.prepare(ctx, dir_mlp, D, false, s);
     if (st == FNR_OK) {
         directions_kernel<<<unsigned((n_rays + 127) / 128), 128, 0, s>>>(F, static_cast<float *>(dirs.p));
         if ((e = cudaGetLastError()) != cudaSuccess) st = cuda_fail(e, "ray directions");
     }
     if (st == FNR_OK)
-        st = dir.launch(static_cast<const float *>(dirs.p), n_rays, nullptr, static_cast<float *>(dir_out.p),
-                        ctx->num_sms, s);
+        st = dir.launch(static_cast<const float *>(dirs.p), n_rays, nullptr, static_cast<float *>(dir_out.p), s);
     for (long long i = 0; i < n_batches && st == FNR_OK; ++i) {
         const int ray0 = int(i * batch), n = int(std::min(batch, n_rays - i * batch));
         unsigned long long *total = static_cast<unsigned long long *>(totals.p) + i;
@@ -287,7 +279,7 @@ extern "C" fnr_status fnr_render_mlp(fnr_context *ctx, const fnr_mlp *pos_mlp, c
             break;
         }
         st = pos.launch(static_cast<const float *>(points.p), (long long)n * rc.N, total,
-                        static_cast<float *>(pos_out.p), ctx->num_sms, s);
+                        static_cast<float *>(pos_out.p), s);
         if (st == FNR_OK &&
             (e = composite(D, F, rc, b, ray0, n, static_cast<const float *>(pos_out.p),
                            static_cast<const float *>(dir_out.p), static_cast<const long long *>(offset.p), s)) !=
