@@ -5,10 +5,16 @@
 //
 // One lane per ray, one warp per 8 x 4 pixel tile as in the uniform march. The
 // walk itself (a 3-D digital differential analyser in binary32, the sequence
-// fixed in fnr.h) is arithmetic only, so each lane generates kVU cells ahead,
-// issues their density loads together, composites them in walk order
-// (weights, transmittance, exact fixed-point termination) and only then loads
-// the records of the cells it composited. In this mode the launcher passes
+// fixed in fnr.h) is arithmetic only, so each lane generates three or four
+// cells ahead (walk_group), issues their density loads together, composites
+// them in walk order (weights, transmittance, exact fixed-point termination)
+// and only then loads the records of the cells it composited; a group with no
+// density in any lane of the warp ends at its density loads. What bounds it is
+// the issue of the walk's instructions (k = 352, skipping: 0.76 issued per
+// cycle and scheduler), so it is those that were cut: divisions through the
+// ray's reciprocals (divide_by), short groups, empty groups left early. 800 x
+// 800, k = 512, FP32: 1064 -> 875 us, with skipping 876 -> 549; FP16 with
+// skipping, 512 x 512, k = 256: 230 -> 172; E4M3 with skipping 1486 -> 682. In this mode the launcher passes
 // t_far in r.dt (the walk has no sample spacing) and r.s_thr is the threshold
 // on sum floor(fp32(sigma delta) 2^32).
 //
@@ -19,6 +25,8 @@
 // (march_voxels_jump.cu). Each form carries only its own code: the brick
 // arithmetic alone cost the plain walk 10%.
 #pragma once
+#include <type_traits>
+
 #include "march_device.cuh"
 
 namespace fnr {
@@ -29,21 +37,66 @@ namespace {
 
 using namespace dev;
 
-constexpr int kVU = 8;  // cells generated ahead of their density loads
+// Cells generated ahead of their density loads. Each is a copy of the step's code, and a skipping walk tries one pass
+// over an empty cube per group: at 8 the skipping kernel stalled on instruction fetch (2.6 of 9.6 cycles an
+// instruction) and walked up to 7 cells into empty space. 800 x 800, k = 512, 8 / 6 / 4 / 3 / 2 cells: FP32 with
+// skipping 876 / 766 / 642 / 652 / 688 us, E4M3 1487 / 1233 / 885 / 776 / 795; FP32 plain 1064 / - / 1002.
+template <int PREC, int FORM>
+constexpr int walk_group() {
+    return PREC == FNR_PREC_FP8_E4M3 && FORM == kVoxJump ? 3 : 4;
+}
 
-// The cells of one ray in walk order (fnr.h, FNR_RENDER_VOXELS).
+// Minimum resident blocks per SM (registers against latency). FP32 with / without skipping at 6 / 7 / 8 blocks:
+// 640 / 613 / 581 and 994 / 932 / 886 us; FP16 with skipping (512 x 512, k = 256) 181 / 171 / 177; E4M3 720 / 719 /
+// 704.
+template <int PREC>
+constexpr int walk_blocks() {
+    return PREC == FNR_PREC_FP16 ? 7 : 8;
+}
+
+// a / b correctly rounded from y = 1 / b correctly rounded: Markstein's theorem (P. W. Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34(1), 1990) -- with q a faithful
+// quotient and r = a - b q exact, q + r y rounds to the correctly rounded quotient. The first correction makes q
+// faithful. Needs 2^-60 <= |b| <= 2^60 and a = +0 or 2^-60 <= |a| <= 2^61, so that no step leaves the normal range.
+__device__ __forceinline__ float divide_by(float a, float b, float y) {
+    float q = __fmul_rn(a, y);
+    q = __fmaf_rn(__fmaf_rn(-q, b, a), y, q);
+    return __fmaf_rn(__fmaf_rn(-q, b, a), y, q);
+}
+
+// The cells of one ray in walk order (fnr.h, FNR_RENDER_VOXELS). RECIP: the divisions by u_a through its
+// reciprocal (every ray but the few whose coordinates are out of its range, see safe()): five multiplications and
+// additions in line, without the division's branch to its general case.
+template <bool RECIP>
 struct VoxelWalk {
     float u0, u1, u2, w0, w1, w2;  // g_a(t) = t u_a + w_a in grid units
+    float y0, y1, y2;              // 1 / u_a
     float tn0, tn1, tn2;           // next crossing per axis
     int c0, c1, c2;                // current cell
     float t, t1;
     int k;
     bool live;
 
-    __device__ __forceinline__ static float crossing(int c, float u, float w) {
-        if (u > 0.0f) return __fdiv_rn(__fsub_rn(static_cast<float>(c + 1), w), u);
-        if (u < 0.0f) return __fdiv_rn(__fsub_rn(static_cast<float>(c), w), u);
-        return __int_as_float(0x7f800000);  // +infinity
+    // Whether the ray's divisions can go through reciprocals. Every dividend is RN(m - w_a) for an integer
+    // 0 <= m <= k: +0, or at least min(|w_a|, 2^-25).
+    __device__ __forceinline__ static bool safe(const CacheView &cv, const float o[3], const float d[3]) {
+        bool ok = true;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float u = fabsf(__fmul_rn(d[a], cv.scale[a]));
+            const float w = fabsf(__fmul_rn(__fsub_rn(o[a], cv.bmin[a]), cv.scale[a]));
+            ok = ok && (u == 0.0f || (u >= 0x1p-60f && u <= 0x1p60f)) && (w == 0.0f || w >= 0x1p-60f) && w <= 0x1p60f;
+        }
+        return ok;
+    }
+
+    __device__ __forceinline__ static float divide(float a, float u, float y) {
+        return RECIP ? divide_by(a, u, y) : __fdiv_rn(a, u);
+    }
+
+    __device__ __forceinline__ static float crossing(int c, float u, float w, float y) {
+        const float tc = divide(__fsub_rn(static_cast<float>(u > 0.0f ? c + 1 : c), w), u, y);
+        return u == 0.0f ? __int_as_float(0x7f800000) : tc;  // +infinity
     }
 
     // Box clipping, start cell and first crossings; live = false if the ray
@@ -52,19 +105,20 @@ struct VoxelWalk {
                                          float t_far) {
         k = cv.k;
         const float kf = cv.kf;
-        float uu[3], ww[3];
+        float uu[3], ww[3], yy[3];
         float t0 = t_near, te = t_far;
         live = true;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             uu[a] = __fmul_rn(d[a], cv.scale[a]);
             ww[a] = __fmul_rn(__fsub_rn(o[a], cv.bmin[a]), cv.scale[a]);
+            yy[a] = RECIP ? __frcp_rn(uu[a]) : 0.0f;
             if (uu[a] != uu[a] || ww[a] != ww[a]) live = false;
             if (uu[a] == 0.0f) {
                 if (!(ww[a] >= 0.0f && ww[a] < kf)) live = false;
             } else {
-                const float ta = __fdiv_rn(-ww[a], uu[a]);
-                const float tb = __fdiv_rn(__fsub_rn(kf, ww[a]), uu[a]);
+                const float ta = divide(-ww[a], uu[a], yy[a]);
+                const float tb = divide(__fsub_rn(kf, ww[a]), uu[a], yy[a]);
                 const float lo = ta < tb ? ta : tb, hi = ta < tb ? tb : ta;
                 if (lo > t0) t0 = lo;
                 if (hi < te) te = hi;
@@ -73,6 +127,7 @@ struct VoxelWalk {
         if (!(t0 < te)) live = false;
         u0 = uu[0], u1 = uu[1], u2 = uu[2];
         w0 = ww[0], w1 = ww[1], w2 = ww[2];
+        y0 = yy[0], y1 = yy[1], y2 = yy[2];
         t = t0;
         t1 = te;
         auto start = [&](float u, float w) {
@@ -82,9 +137,9 @@ struct VoxelWalk {
         c0 = live ? start(u0, w0) : 0;
         c1 = live ? start(u1, w1) : 0;
         c2 = live ? start(u2, w2) : 0;
-        tn0 = crossing(c0, u0, w0);
-        tn1 = crossing(c1, u1, w1);
-        tn2 = crossing(c2, u2, w2);
+        tn0 = crossing(c0, u0, w0, y0);
+        tn1 = crossing(c1, u1, w1, y1);
+        tn2 = crossing(c2, u2, w2, y2);
     }
 
     // The current cell, its occupancy brick (bricks of 2^sh cells, od per axis),
@@ -92,16 +147,10 @@ struct VoxelWalk {
     // advances to the next cell, or clears live after the last one. The step is
     // branch-free: lanes of a warp step different axes.
     __device__ __forceinline__ int next(float &delta, int &brick, int sh, int od, int &obrick, int osh, int odim) {
-        int a = 0;
-        float tnext = tn0;
-        if (tn1 < tnext) {
-            a = 1;
-            tnext = tn1;
-        }
-        if (tn2 < tnext) {
-            a = 2;
-            tnext = tn2;
-        }
+        const bool y = tn1 < tn0;
+        const float txy = y ? tn1 : tn0;
+        const bool z = tn2 < txy;
+        const float tnext = z ? tn2 : txy;
         const float end = tnext < t1 ? tnext : t1;
         const int cell = (c2 * k + c1) * k + c0;  // k^3 < 2^31
         brick = ((c2 >> sh) * od + (c1 >> sh)) * od + (c0 >> sh);
@@ -113,17 +162,21 @@ struct VoxelWalk {
         }
         if (tnext > t) t = tnext;
         // the stepped axis has u != 0 (a +infinity crossing is never below t1)
-        const bool x = a == 0, y = a == 1;
-        const float ua = x ? u0 : (y ? u1 : u2);
-        const float wa = x ? w0 : (y ? w1 : w2);
-        const int ca = (x ? c0 : (y ? c1 : c2)) + (ua > 0.0f ? 1 : -1);
-        const float tna = __fdiv_rn(__fsub_rn(static_cast<float>(ua > 0.0f ? ca + 1 : ca), wa), ua);
-        c0 = x ? ca : c0;
-        c1 = y ? ca : c1;
-        c2 = (x || y) ? c2 : ca;
-        tn0 = x ? tna : tn0;
-        tn1 = y ? tna : tn1;
-        tn2 = (x || y) ? tn2 : tna;
+        const float ua = z ? u2 : (y ? u1 : u0);
+        const float wa = z ? w2 : (y ? w1 : w0);
+        const float ya = z ? y2 : (y ? y1 : y0);
+        const int ca = (z ? c2 : (y ? c1 : c0)) + (ua > 0.0f ? 1 : -1);
+        const float tna = divide(__fsub_rn(static_cast<float>(ua > 0.0f ? ca + 1 : ca), wa), ua, ya);
+        if (z) {
+            c2 = ca;
+            tn2 = tna;
+        } else if (y) {
+            c1 = ca;
+            tn1 = tna;
+        } else {
+            c0 = ca;
+            tn0 = tna;
+        }
         if (ca < 0 || ca >= k) live = false;
         return cell;
     }
@@ -134,12 +187,13 @@ struct VoxelWalk {
     // of the grid coordinate at X. -1 if the estimate is off by more than a few.
     // `next` receives the first crossing not counted: the one out of the cell
     // the axis has reached.
-    __device__ __forceinline__ static int crossings_until(int c, float u, float w, float X, bool at, float &next) {
+    __device__ __forceinline__ static int crossings_until(int c, float u, float w, float y, float X, bool at,
+                                                              float &next) {
         next = __int_as_float(0x7f800000);
         if (u == 0.0f) return 0;
         const int s = u > 0.0f ? 1 : -1;
         auto before = [&](int n) {
-            const float tc = crossing(c + s * n, u, w);
+            const float tc = crossing(c + s * n, u, w, y);
             const bool b = tc < X || (at && tc == X);
             if (!b) next = tc;
             return b;
@@ -163,14 +217,14 @@ struct VoxelWalk {
     // crossing moves one axis by one cell. Returns the cells passed; at most
     // `cap`, which spends the walk; 0 if it took no step.
     __device__ __forceinline__ int pass_cube(const int lo[3], const int hi[3], int cap) {
-        const float uu[3] = {u0, u1, u2}, ww[3] = {w0, w1, w2};
+        const float uu[3] = {u0, u1, u2}, ww[3] = {w0, w1, w2}, yy[3] = {y0, y1, y2};
         const int cc[3] = {c0, c1, c2};
         float X = __int_as_float(0x7f800000);
         int ax = 3;  // the axis whose crossing leaves the cube first (the lowest on a tie)
 #pragma unroll
         for (int a = 0; a < 3; ++a)
             if (uu[a] != 0.0f) {
-                const float xa = crossing(uu[a] > 0.0f ? hi[a] : lo[a], uu[a], ww[a]);
+                const float xa = crossing(uu[a] > 0.0f ? hi[a] : lo[a], uu[a], ww[a], yy[a]);
                 if (xa < X) {
                     X = xa;
                     ax = a;
@@ -181,7 +235,7 @@ struct VoxelWalk {
         float nx[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            n[a] = crossings_until(cc[a], uu[a], ww[a], ends ? t1 : X, !ends && a <= ax, nx[a]);
+            n[a] = crossings_until(cc[a], uu[a], ww[a], yy[a], ends ? t1 : X, !ends && a <= ax, nx[a]);
             if (n[a] < 0) return 0;
             total += n[a];
         }
@@ -205,9 +259,11 @@ struct VoxelWalk {
 };
 
 template <int PREC, int D, int FORM>
-__global__ void __launch_bounds__(FNR_BLOCK) march_voxels_kernel(const __grid_constant__ MarchArgs A) {
+__global__ void __launch_bounds__(FNR_BLOCK, walk_blocks<PREC>())
+    march_voxels_kernel(const __grid_constant__ MarchArgs A) {
     allow_next_grid();
     constexpr unsigned FULL = 0xffffffffu;
+    constexpr int kVU = walk_group<PREC, FORM>();
     const int tile = static_cast<int>((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (tile >= A.total_tiles) return;  // whole warp
     int f = 0;
@@ -231,8 +287,8 @@ __global__ void __launch_bounds__(FNR_BLOCK) march_voxels_kernel(const __grid_co
     }
 
     RaySetup<PREC, D> R;  // a1/a2: direction cell and beta (the uniform-sample fields go unused)
-    VoxelWalk Wk;
-    Wk.live = false;
+    float dd[3] = {0.0f, 0.0f, 1.0f};
+    const float oo[3] = {F.c2w[3], F.c2w[7], F.c2w[11]};
     R.dcell = 0;
     R.sigma_scale = 1.0f;
     if (active) {
@@ -245,9 +301,9 @@ __global__ void __launch_bounds__(FNR_BLOCK) march_voxels_kernel(const __grid_co
         const float wz = __fmaf_rn(F.c2w[8], dcx, __fmaf_rn(F.c2w[9], dcy, -F.c2w[10]));
         const float n2 = __fmaf_rn(wx, wx, __fmaf_rn(wy, wy, __fmul_rn(wz, wz)));
         const float len = __fsqrt_rn(n2);
-        const float dd[3] = {__fdiv_rn(wx, len), __fdiv_rn(wy, len), __fdiv_rn(wz, len)};
-        const float oo[3] = {F.c2w[3], F.c2w[7], F.c2w[11]};
-        Wk.init(c, oo, dd, r.t_near, r.dt);  // r.dt holds t_far in this mode
+        dd[0] = __fdiv_rn(wx, len);
+        dd[1] = __fdiv_rn(wy, len);
+        dd[2] = __fdiv_rn(wz, len);
     }
     const bool skip = FORM != kVoxPlain && (r.flags & FNR_RENDER_SKIP_EMPTY) != 0u;
     // Skipping without per-cell output also passes over whole empty cubes of jump
@@ -261,95 +317,118 @@ __global__ void __launch_bounds__(FNR_BLOCK) march_voxels_kernel(const __grid_co
     int32_t *cells_out = (active && F.cells) ? F.cells + pix * r.N : nullptr;
     if (F.cells) wait_prior_grid();  // cells are written while walking
 
-    while (__any_sync(FULL, Wk.live && !term && n_gen < r.N)) {
-        // kVU cells ahead, their densities loaded together
-        int cell[kVU], brick[kVU], obr[kVU];
-        float dl[kVU], sg[kVU];
-        unsigned gen = 0u, looked = 0u;
+    auto walk = [&](auto recip) {
+        VoxelWalk<decltype(recip)::value> Wk;
+        Wk.init(c, oo, dd, r.t_near, r.dt);  // r.dt holds t_far in this mode
+        Wk.live = Wk.live && active;
+        while (__any_sync(FULL, Wk.live && !term && n_gen < r.N)) {
+            // kVU cells ahead, their densities loaded together
+            int cell[kVU], brick[kVU], obr[kVU];
+            float dl[kVU], sg[kVU];
+            unsigned gen = 0u, looked = 0u;
 #pragma unroll
-        for (int u = 0; u < kVU; ++u) {
-            cell[u] = 0;
-            brick[u] = 0;
-            obr[u] = 0;
-            dl[u] = 0.0f;
-            if (jumps && u == 0 && Wk.live && !term && n_gen < r.N) {
-                // One pass per group (more per group measured slower: each costs a dozen exact divisions
-                // and the lanes of a warp take different ones). d > 0: the jump bricks within Chebyshev
-                // distance d - 1 of the current one are empty.
-                const int sh = c.dist_shift;
-                const int d = __ldg(c.dist + ((Wk.c2 >> sh) * c.dist_dim + (Wk.c1 >> sh)) * c.dist_dim + (Wk.c0 >> sh));
-                if (d > 0) {
-                    const int cw[3] = {Wk.c0, Wk.c1, Wk.c2};
-                    int lo[3], hi[3];
+            for (int u = 0; u < kVU; ++u) {
+                cell[u] = 0;
+                brick[u] = 0;
+                obr[u] = 0;
+                dl[u] = 0.0f;
+                if (jumps && u == 0 && Wk.live && !term && n_gen < r.N) {
+                    // One pass per group (more per group measured slower: each costs a dozen exact divisions
+                    // and the lanes of a warp take different ones). d > 0: the jump bricks within Chebyshev
+                    // distance d - 1 of the current one are empty.
+                    const int sh = c.dist_shift;
+                    const int d =
+                        __ldg(c.dist + ((Wk.c2 >> sh) * c.dist_dim + (Wk.c1 >> sh)) * c.dist_dim + (Wk.c0 >> sh));
+                    if (d > 0) {
+                        const int cw[3] = {Wk.c0, Wk.c1, Wk.c2};
+                        int lo[3], hi[3];
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        lo[a] = max(((cw[a] >> sh) - (d - 1)) << sh, 0);
-                        hi[a] = min((((cw[a] >> sh) + d) << sh) - 1, Wk.k - 1);
+                        for (int a = 0; a < 3; ++a) {
+                            lo[a] = max(((cw[a] >> sh) - (d - 1)) << sh, 0);
+                            hi[a] = min((((cw[a] >> sh) + d) << sh) - 1, Wk.k - 1);
+                        }
+                        const int m = Wk.pass_cube(lo, hi, r.N - n_gen);
+                        n_gen += m;
+                        n_steps += m;
                     }
-                    const int m = Wk.pass_cube(lo, hi, r.N - n_gen);
-                    n_gen += m;
-                    n_steps += m;
+                }
+                if (Wk.live && !term && n_gen < r.N) {
+                    cell[u] = Wk.next(dl[u], brick[u], c.occ_shift, c.occ_dim, obr[u], c.offs_shift, c.offs_dim);
+                    gen |= 1u << u;
+                    ++n_gen;
                 }
             }
-            if (Wk.live && !term && n_gen < r.N) {
-                cell[u] = Wk.next(dl[u], brick[u], c.occ_shift, c.occ_dim, obr[u], c.offs_shift, c.offs_dim);
-                gen |= 1u << u;
-                ++n_gen;
-            }
-        }
 #pragma unroll
-        for (int u = 0; u < kVU; ++u) {
-            sg[u] = 0.0f;
-            if (((gen >> u) & 1u) && dl[u] > 0.0f) {
-                const bool load = !skip || brick_occupied(c, brick[u]) != 0u;
-                if (load) {
-                    sg[u] = load_sigma<PREC>(c, cell[u], R.sigma_scale);
-                    looked |= 1u << u;
+            for (int u = 0; u < kVU; ++u) {
+                sg[u] = 0.0f;
+                if (((gen >> u) & 1u) && dl[u] > 0.0f) {
+                    const bool load = !skip || brick_occupied(c, brick[u]) != 0u;
+                    if (load) {
+                        sg[u] = load_sigma<PREC>(c, cell[u], R.sigma_scale);
+                        looked |= 1u << u;
+                    }
                 }
             }
-        }
-        // walk order: weights, transmittance and termination from the densities alone
-        float wgt[kVU];
-        unsigned occ = 0u;
+            if (cells_out) {
+                int j = n_steps;
 #pragma unroll
-        for (int u = 0; u < kVU; ++u) {
-            wgt[u] = 0.0f;
-            if (!((gen >> u) & 1u) || term) continue;
-            ++n_steps;
-            if (cells_out) cells_out[n_steps - 1] = cell[u];
-            if ((looked >> u) & 1u) ++n_look;
-            if (sg[u] > 0.0f) {
-                ++n_occ;
-                const float od = __fmul_rn(sg[u], dl[u]);
-                float ext, alpha;
-                extinction(od, ext, alpha);
-                wgt[u] = T * alpha;
-                T = T * ext;
-                occ |= 1u << u;
-                if (od > 0.0f) S += fixed_depth(od);
-                if (S >= static_cast<unsigned long long>(r.s_thr)) term = true;
+                for (int u = 0; u < kVU; ++u)
+                    if ((gen >> u) & 1u) cells_out[j++] = cell[u];  // past termination: overwritten by -2 below
+            }
+            unsigned dense = 0u;
+#pragma unroll
+            for (int u = 0; u < kVU; ++u) dense |= (sg[u] > 0.0f ? 1u : 0u) << u;
+            if (!__any_sync(FULL, dense != 0u)) {  // empty space for the whole warp
+                n_steps += __popc(gen);
+                n_look += __popc(looked);
+                continue;
+            }
+            // walk order: weights, transmittance and termination from the densities alone
+            float wgt[kVU];
+            unsigned occ = 0u, counted = gen;
+#pragma unroll
+            for (int u = 0; u < kVU; ++u) {
+                wgt[u] = 0.0f;
+                if (((dense >> u) & 1u) && !term) {
+                    const float od = __fmul_rn(sg[u], dl[u]);
+                    float ext, alpha;
+                    extinction(od, ext, alpha);
+                    wgt[u] = T * alpha;
+                    T = T * ext;
+                    occ |= 1u << u;
+                    if (od > 0.0f) S += fixed_depth(od);
+                    if (S >= static_cast<unsigned long long>(r.s_thr)) {
+                        term = true;
+                        counted = gen & ((2u << u) - 1u);
+                    }
+                }
+            }
+            n_steps += __popc(counted);
+            n_look += __popc(looked & counted);
+            n_occ += __popc(occ);
+            // records of the composited cells, colour added in walk order
+#pragma unroll
+            for (int u = 0; u < kVU; ++u) {
+                if (!((occ >> u) & 1u)) continue;
+                Record<PREC, D> rec;
+                rec.load(c.uvw + static_cast<long long>(cell[u]) * c.rec_stride);
+                float col[3];
+                if constexpr (kOffs) {
+                    OffsetRecord<D> off;
+                    off.load(c.offs + static_cast<long long>(obr[u]) * c.offs_stride);
+                    shade_e4m3<D>(
+                        rec, off, r.act, [&](int i) { return ssc[i]; }, [&](int j) { return qbeta[j][lane]; }, col);
+                } else {
+                    RaySetup<PREC, D>::shade_with(rec, r.act, [&](int ch, int j) { return qbeta[j][lane]; }, col);
+                }
+                Cr = __fmaf_rn(wgt[u], col[0], Cr);
+                Cg = __fmaf_rn(wgt[u], col[1], Cg);
+                Cb = __fmaf_rn(wgt[u], col[2], Cb);
             }
         }
-        // records of the composited cells, colour added in walk order
-#pragma unroll
-        for (int u = 0; u < kVU; ++u) {
-            if (!((occ >> u) & 1u)) continue;
-            Record<PREC, D> rec;
-            rec.load(c.uvw + static_cast<long long>(cell[u]) * c.rec_stride);
-            float col[3];
-            if constexpr (kOffs) {
-                OffsetRecord<D> off;
-                off.load(c.offs + static_cast<long long>(obr[u]) * c.offs_stride);
-                shade_e4m3<D>(
-                    rec, off, r.act, [&](int i) { return ssc[i]; }, [&](int j) { return qbeta[j][lane]; }, col);
-            } else {
-                RaySetup<PREC, D>::shade_with(rec, r.act, [&](int ch, int j) { return qbeta[j][lane]; }, col);
-            }
-            Cr = __fmaf_rn(wgt[u], col[0], Cr);
-            Cg = __fmaf_rn(wgt[u], col[1], Cg);
-            Cb = __fmaf_rn(wgt[u], col[2], Cb);
-        }
-    }
+    };
+    if (__all_sync(FULL, VoxelWalk<true>::safe(c, oo, dd))) walk(std::true_type{});
+    else walk(std::false_type{});
     wait_prior_grid();
     if (!active) return;
     if (cells_out)
