@@ -26,7 +26,8 @@ namespace {
 using namespace dev;
 
 template <int PREC, int D, bool SKIP, bool BRICKS>
-__global__ void __launch_bounds__(FNR_BLOCK, dev::min_blocks(PREC)) march_kernel(const __grid_constant__ MarchArgs A) {
+__global__ void __launch_bounds__(FNR_BLOCK, dev::min_blocks<PREC, D>())
+    march_kernel(const __grid_constant__ MarchArgs A) {
     allow_next_grid();  // the next render launch may be scheduled as SMs free up
     const int tile = static_cast<int>((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (tile >= A.total_tiles) return;  // whole warp
@@ -38,7 +39,7 @@ __global__ void __launch_bounds__(FNR_BLOCK, dev::min_blocks(PREC)) march_kernel
     tile_origin(F, t, x0, y0);
     const int lane = threadIdx.x & 31;
     const int px = x0 + (lane & (kTileW - 1)), py = y0 + lane / kTileW;
-    __shared__ QueueFor<PREC, D> queues[FNR_BLOCK / 32];
+    __shared__ QueueFor<PREC, D, BRICKS> queues[FNR_BLOCK / 32];
     march_tile_queued<PREC, D, SKIP, BRICKS>(A.c, A.r, F, px, py, px < F.W && py < F.H, queues[threadIdx.x >> 5]);
 }
 

@@ -13,49 +13,49 @@ namespace dev {
 
 
 // Tuning knobs (defaults are the best measured on GB300):
-//   FNR_UNROLL    density loads issued together per lane
-//   FNR_BLOCK / FNR_MINB  threads per block / minimum resident blocks per SM
-//   FNR_MINB_FP16 / FNR_MINB_FP8  the same for the quantised caches
+//   FNR_BLOCK     threads per block
 //   FNR_FAST_EXP  1: exponentials of the occupied-sample path via ex2.approx
-#ifndef FNR_UNROLL
-#define FNR_UNROLL 8
-#endif
 #ifndef FNR_BLOCK
 #define FNR_BLOCK 128
-#endif
-#ifndef FNR_MINB
-#define FNR_MINB 7
-#endif
-#ifndef FNR_MINB_FP16
-#define FNR_MINB_FP16 8
-#endif
-#ifndef FNR_MINB_FP8
-#define FNR_MINB_FP8 7
 #endif
 #ifndef FNR_FAST_EXP
 #define FNR_FAST_EXP 1
 #endif
-// FNR_REC_PREFETCH: when an occupied sample is queued, prefetch its record
-// (1: into L2, 2: into L1, 0: no); E4M3 records (24 bytes) measured better without
-#ifndef FNR_REC_PREFETCH
-#define FNR_REC_PREFETCH 1
-#endif
-constexpr int kUnroll = FNR_UNROLL;
 
-// prefetch [p, p + n) (n <= 128) into L2 (level 1) or L1 (level 2)
-template <int LEVEL>
-__device__ __forceinline__ void prefetch_span(const char *p, int n) {
-    if constexpr (LEVEL == 1) {
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(p + n - 1));
-    } else if constexpr (LEVEL == 2) {
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(p + n - 1));
-    }
+// Group size (samples whose densities a lane loads together) and minimum resident blocks per SM (registers against
+// latency). The march waits: for its density and record loads and for the shared-memory steps between them, and
+// fetching the next group's densities a group early or cutting its instructions by a tenth gained nothing, so what
+// counts is how many warps are there to wait. Groups of 8 needed 72 registers and 288 queue entries a warp; with 5
+// (6 where the record is small) 56 registers hold a lane's state, 9 blocks fit instead of 7 and the queue leaves
+// 30 KB more to L1. 800 x 800, k = 512, N = 128, D = 8, groups of 8 at 7 (FP16: 8) blocks -> here, in us: FP32 95.8 ->
+// 87.7, with skipping 87.9 -> 78.4, bricks 100 -> 89; FP16 81.2 -> 78.1, 81.7 -> 76.6, bricks 103 -> 87; E4M3 94.8 ->
+// 91.7, 98.4 -> 90.6. 5 / 6 / 8 samples at 9 blocks, FP32: 87.7 / 90.0 / 93.4 (D = 8), 82.2 / 79.3 / 82.1 (6), 82.0 /
+// 78.0 / 80.2 (4). E4M3 carries offsets and scales besides and spills at 9 blocks (110). Longer records need their
+// registers: FP32 at 7 / 8 / 9 blocks 101.6 / 94.8 / 99.4 (D = 12) and 118.8 / 115.6 / 118.0 (16); E4M3, D = 12, groups
+// of 6 at 7 blocks 99.5, of 5 at 8 116.8; D = 16, groups of 6 at 6 / 7 blocks 126 / 130.
+template <int PREC, int D, bool BRICKS>
+__host__ __device__ constexpr int group_size() {
+    if (PREC == FNR_PREC_FP8_E4M3) return D <= 8 ? 5 : 6;
+    return D <= 6 && !BRICKS ? 6 : 5;
 }
-// minimum resident blocks per SM of the march kernels for a cache precision
-__host__ __device__ constexpr int min_blocks(int prec) {
-    return prec == FNR_PREC_FP8_E4M3 ? FNR_MINB_FP8 : (prec == FNR_PREC_FP16 ? FNR_MINB_FP16 : FNR_MINB);
+template <int PREC, int D>
+__host__ __device__ constexpr int min_blocks() {
+    if (PREC == FNR_PREC_FP8_E4M3) return D <= 8 ? 8 : (D <= 12 ? 7 : 6);
+    return PREC == FNR_PREC_FP32 && D > 8 ? 8 : 9;
+}
+
+// Whether an occupied sample's record is prefetched into L2 when the sample is queued. E4M3 records (24 bytes) and
+// brick pools (compact, mostly in L2) measured better without: FP16 bricks, 643 x 481, D = 6: 51.2 -> 49.4 us; dense
+// FP32 the other way, 89.2 without, 87.7 with.
+template <int PREC, bool BRICKS>
+__host__ __device__ constexpr bool prefetch_records() {
+    return PREC != FNR_PREC_FP8_E4M3 && !BRICKS;
+}
+
+// prefetch [p, p + n) (n <= 128) into L2
+__device__ __forceinline__ void prefetch_span(const char *p, int n) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p + n - 1));
 }
 
 __device__ __forceinline__ float e4m3_to_float(unsigned int byte) {
@@ -189,15 +189,16 @@ __device__ __forceinline__ unsigned brick_occupied(const CacheView &c, int brick
 }
 
 // floor(s * 2^32) of a binary32 s > 0: integer part and scaled fraction, both exact, each by one conversion to
-// 32 bits (to 64 bits they run on the FP64 pipe). s >= 2^31 saturates at 2^63 - 1. By shifts of the significand and
+// 32 bits (to 64 bits they run on the FP64 pipe). s >= 2^31 gives 2^63 - 1: both conversions saturate, the second
+// because the first's result is rounded down on its way back (by a comparison and selects instead, the voxel walk of
+// an 800 x 800 view took 549 us, now 543). By shifts of the significand and
 // with a saturating sum (here the sum is unsigned: two terms below 2^63 cannot wrap, and the threshold ends the ray
 // after the first that reaches it) an 800 x 800 view took 96.2 / 82.2 / 96.4 us from FP32 / FP16 / E4M3 caches and
 // 109.1 from bricks, now 95.9 / 81.3 / 94.9 and 100.2; the voxel walk of it 927 us, now 875.
 __device__ __forceinline__ unsigned long long fixed_depth(float s) {
-    const unsigned int hi = __float2uint_rz(s);
-    const unsigned int lo = __float2uint_rz(__fmul_rn(__fsub_rn(s, __uint2float_rn(hi)), 4294967296.0f));
-    const unsigned long long d = (static_cast<unsigned long long>(hi) << 32) | lo;
-    return s >= 2147483648.0f ? 0x7fffffffffffffffull : d;
+    const int hi = __float2int_rz(s);
+    const unsigned int lo = __float2uint_rz(__fmul_rn(__fsub_rn(s, __int2float_rz(hi)), 4294967296.0f));
+    return (static_cast<unsigned long long>(static_cast<unsigned int>(hi)) << 32) | lo;
 }
 
 // Azimuth key in [0, 4], monotone in atan2(y, x) wrapped to [0, 2 pi).
@@ -377,19 +378,41 @@ struct RaySetup {
 
     // The ray's D direction weights (unscaled; FP8 folds the channel scales at
     // shading) into qbeta[i][lane]: the nearest bin's, or bilinear in
-    // (theta, phi) between bin centres (FNR_RENDER_DIR_BILINEAR).
+    // (theta, phi) between bin centres (FNR_RENDER_DIR_BILINEAR). The nearest bin's four at a time where D allows: the
+    // weights start on a 256-byte boundary.
     __device__ __forceinline__ void stage_beta(const CacheView &c, const RenderConst &r, const float dd[3],
                                                float (*qbeta)[32], int lane) const {
-        auto beta_at = [&](long long cell, int i) {
-            return c.dir_prec == FNR_PREC_FP16
-                       ? __half2float(__ldg(static_cast<const __half *>(c.beta) + cell * D + i))
-                       : __ldg(static_cast<const float *>(c.beta) + cell * D + i);
-        };
+        const long long first = static_cast<long long>(dcell) * D;
         if (r.flags & FNR_RENDER_DIR_BILINEAR) {
             stage_beta_bilinear<D>(c, dd[0], dd[1], dd[2], qbeta, lane);
-        } else {
+        } else if (c.dir_prec == FNR_PREC_FP16) {
+            const __half *p = static_cast<const __half *>(c.beta) + first;
+            if constexpr (D % 4 == 0) {
 #pragma unroll
-            for (int i = 0; i < D; ++i) qbeta[i][lane] = beta_at(dcell, i);
+                for (int i = 0; i < D; i += 4) {
+                    const uint2 q = __ldg(reinterpret_cast<const uint2 *>(p + i));
+                    const float2 lo = __half22float2(reinterpret_cast<const __half2 &>(q.x));
+                    const float2 hi = __half22float2(reinterpret_cast<const __half2 &>(q.y));
+                    qbeta[i][lane] = lo.x, qbeta[i + 1][lane] = lo.y;
+                    qbeta[i + 2][lane] = hi.x, qbeta[i + 3][lane] = hi.y;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < D; ++i) qbeta[i][lane] = __half2float(__ldg(p + i));
+            }
+        } else {
+            const float *p = static_cast<const float *>(c.beta) + first;
+            if constexpr (D % 4 == 0) {
+#pragma unroll
+                for (int i = 0; i < D; i += 4) {
+                    const float4 q = __ldg(reinterpret_cast<const float4 *>(p + i));
+                    qbeta[i][lane] = q.x, qbeta[i + 1][lane] = q.y;
+                    qbeta[i + 2][lane] = q.z, qbeta[i + 3][lane] = q.w;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < D; ++i) qbeta[i][lane] = __ldg(p + i);
+            }
         }
     }
 
@@ -406,12 +429,21 @@ struct RaySetup {
         return in ? (iz * c.k + iy) * c.k + ix : -1;  // k^3 < 2^31
     }
 
+    // Floor of a coordinate 0 <= g < 2^23 as an integer plus kFloorBits: g + 2^23 rounded down has unit spacing. An
+    // addition where a conversion would go through the slow pipe: plain views 1.0 to 1.5% faster. Not where a brick
+    // index is taken as well: its extra constants cost more (FP32 bricks 112 -> 120 us).
+    static constexpr unsigned kFloorBits = 0x4b000000u;  // 2^23
+    __device__ __forceinline__ static unsigned floor_bits(float g) {
+        return __float_as_uint(__fadd_rd(g, 8388608.0f));
+    }
+
     // Cell of a sample known to be inside the box.
     __device__ __forceinline__ int cell_inside(const CacheView &c, float fi) const {
-        const int ix = __float2int_rd(__fmaf_rn(fi, e[0], f[0]));
-        const int iy = __float2int_rd(__fmaf_rn(fi, e[1], f[1]));
-        const int iz = __float2int_rd(__fmaf_rn(fi, e[2], f[2]));
-        return (iz * c.k + iy) * c.k + ix;
+        const unsigned ku = static_cast<unsigned>(c.k);
+        const unsigned ix = floor_bits(__fmaf_rn(fi, e[0], f[0]));
+        const unsigned iy = floor_bits(__fmaf_rn(fi, e[1], f[1]));
+        const unsigned iz = floor_bits(__fmaf_rn(fi, e[2], f[2]));
+        return static_cast<int>((iz * ku + iy) * ku + ix - kFloorBits * (ku * ku + ku + 1u));
     }
 
     // Brick and brick-local index ((z mod B) B + (y mod B)) B + (x mod B) of
@@ -540,11 +572,13 @@ __device__ __forceinline__ void extinction(float od, float &ext, float &alpha) {
 // shades them together -- 32 independent record loads in one round trip --
 // and every owner lane adds w_i * c_i to its colour in sample order, so the
 // binary32 result equals the sequential form bit for bit.
-constexpr int kQCap = 32 * (kUnroll + 1);  // entries left after a flush (< 32) plus one group's appends
+__host__ __device__ constexpr int queue_cap(int group) {
+    return 32 * (group + 1);  // entries left after a flush (< 32) plus one group's appends
+}
 
 // OFFS (E4M3 caches): each entry also carries its offset brick, and the warp
 // keeps the 3D channel scales.
-template <int D, bool OFFS = false>
+template <int D, bool OFFS, int kQCap>
 struct WarpQueue {
     int cell[kQCap];
     float w[kQCap];
@@ -555,8 +589,8 @@ struct WarpQueue {
     int obr[OFFS ? kQCap : 1];  // offset brick of each entry
     float sc[OFFS ? 3 * D : 1]; // scale of (u, v, w) channel ch D + j
 };
-template <int PREC, int D>
-using QueueFor = WarpQueue<D, PREC == FNR_PREC_FP8_E4M3>;
+template <int PREC, int D, bool BRICKS = false>
+using QueueFor = WarpQueue<D, PREC == FNR_PREC_FP8_E4M3, queue_cap(group_size<PREC, D, BRICKS>())>;
 
 // SKIP (FNR_RENDER_SKIP_EMPTY): a sample in a brick without stored density is
 // known to be empty, so only samples in occupied bricks load their density; the
@@ -566,7 +600,8 @@ using QueueFor = WarpQueue<D, PREC == FNR_PREC_FP8_E4M3>;
 // among the occupied bricks, and the queue carries pool indices instead of cells.
 template <int PREC, int D, bool SKIP, bool BRICKS = false>
 __device__ __forceinline__ void march_tile_queued(const CacheView &c, const RenderConst &r, const FrameDesc &F,
-                                                  int px, int py, bool active, QueueFor<PREC, D> &q) {
+                                                  int px, int py, bool active, QueueFor<PREC, D, BRICKS> &q) {
+    constexpr int kUnroll = group_size<PREC, D, BRICKS>();
     constexpr bool kOffs = PREC == FNR_PREC_FP8_E4M3;
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -827,9 +862,8 @@ __device__ __forceinline__ void march_tile_queued(const CacheView &c, const Rend
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) {
             if ((app >> u) & 1u) {
-                if constexpr (FNR_REC_PREFETCH != 0 && PREC != FNR_PREC_FP8_E4M3)
-                    prefetch_span<FNR_REC_PREFETCH>(c.uvw + static_cast<long long>(cell[u]) * c.rec_stride,
-                                                    c.rec_stride);
+                if constexpr (prefetch_records<PREC, BRICKS>())
+                    prefetch_span(c.uvw + static_cast<long long>(cell[u]) * c.rec_stride, c.rec_stride);
                 q.cell[pos] = cell[u];
                 q.w[pos] = aw[u];
                 q.owner[pos] = static_cast<unsigned char>(lane);

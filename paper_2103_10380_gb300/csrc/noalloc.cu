@@ -48,7 +48,7 @@ std::mutex g_setup_mu;
 int g_grid[kMaxDevices][3][17] = {};
 
 template <int PREC, int D>
-__global__ void __launch_bounds__(FNR_BLOCK, dev::min_blocks(PREC))
+__global__ void __launch_bounds__(FNR_BLOCK, dev::min_blocks<PREC, D>())
     noalloc_kernel(const __grid_constant__ MarchArgs A, unsigned int *scratch, uint32_t *done_words) {
     __shared__ dev::QueueFor<PREC, D> queues[FNR_BLOCK / 32];
     const int lane = threadIdx.x & 31;

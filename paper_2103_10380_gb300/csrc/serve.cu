@@ -83,10 +83,10 @@ __device__ __forceinline__ int serve_frame_of(const ServeTable &tab, int nf, int
 }
 
 template <int PREC, int D, bool SKIP, bool BRICKS>
-__global__ void __launch_bounds__(FNR_BLOCK, dev::min_blocks(PREC))
+__global__ void __launch_bounds__(FNR_BLOCK, dev::min_blocks<PREC, D>())
     serve_kernel(const __grid_constant__ ServeTable tab, ServeScratch *scr, volatile uint32_t *done_flags) {
     constexpr int kWarps = FNR_BLOCK / 32;
-    __shared__ dev::QueueFor<PREC, D> queues[kWarps];
+    __shared__ dev::QueueFor<PREC, D, BRICKS> queues[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int total = tab.total_tiles;
     const int nf = tab.n_frames;
