@@ -13,8 +13,9 @@
 // the issue of the walk's instructions (k = 352, skipping: 0.76 issued per
 // cycle and scheduler), so it is those that were cut: divisions through the
 // ray's reciprocals (divide_by), short groups, empty groups left early. 800 x
-// 800, k = 512, FP32: 1064 -> 875 us, with skipping 876 -> 543; FP16 with
-// skipping, 512 x 512, k = 256: 230 -> 172; E4M3 with skipping 1486 -> 675. In this mode the launcher passes
+// 800, k = 512, FP32: 1064 -> 875 us, with skipping 876 -> 543; FP16,
+// 512 x 512, k = 256: 230 -> 172, with skipping 265 -> 162; E4M3 with skipping
+// 1486 -> 675. In this mode the launcher passes
 // t_far in r.dt (the walk has no sample spacing) and r.s_thr is the threshold
 // on sum floor(fp32(sigma delta) 2^32).
 //
@@ -47,8 +48,8 @@ constexpr int walk_group() {
 }
 
 // Minimum resident blocks per SM (registers against latency). FP32 with / without skipping at 6 / 7 / 8 blocks:
-// 640 / 613 / 581 and 994 / 932 / 886 us; FP16 with skipping (512 x 512, k = 256) 181 / 171 / 177; E4M3 720 / 719 /
-// 704.
+// 640 / 613 / 581 and 994 / 932 / 886 us; FP16 without skipping (512 x 512, k = 256) 181 / 171 / 177; E4M3 with it
+// 720 / 719 / 704.
 template <int PREC>
 constexpr int walk_blocks() {
     return PREC == FNR_PREC_FP16 ? 7 : 8;
