@@ -23,8 +23,10 @@ def sources():
 
 
 def _deps_mtime():
-    files = sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".h")]
-    files.append(os.path.join(ROOT, "include", "fnr.h"))
+    """The newest change of anything the library is made from: sources, every header they include (the kernels
+    themselves live in .cuh files) and this script."""
+    files = [os.path.join(d, f) for d in (CSRC, os.path.join(ROOT, "include")) for f in os.listdir(d)
+             if f.endswith((".cu", ".cuh", ".h"))]
     files.append(os.path.abspath(__file__))
     return max(os.path.getmtime(f) for f in files)
 
