@@ -584,7 +584,7 @@ static fnr_status build_dense(fnr_context *ctx, const fnr_cache_desc *desc, cons
     } else {
         return fail(FNR_ERR_INVALID_ARG, "unknown source kind %d", src->kind);
     }
-    cudaError_t e = use_device(ctx->device);
+    cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_fail(e, "cudaSetDevice");
     const Layout L = layout_of(desc, -1, records);
     const uint64_t charge = layout_of(desc).total;
@@ -758,7 +758,7 @@ fnr_status fnr_cache_load(fnr_context *ctx, const char *path, fnr_stream_t strea
     if (h.footprint != L.total)
         return fail(FNR_ERR_IO, "%s: footprint %llu does not match the descriptor's %llu", path,
                     (unsigned long long)h.footprint, (unsigned long long)L.total);
-    cudaError_t e = use_device(ctx->device);
+    cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_fail(e, "cudaSetDevice");
     if (!budget_charge(ctx, L.total))
         return fail(FNR_ERR_BUDGET, "cache needs %llu bytes, budget %llu, in use %llu", (unsigned long long)L.total,
@@ -847,7 +847,7 @@ fnr_status fnr_render(fnr_context *ctx, const fnr_cache *cache, const fnr_camera
         return fail(FNR_ERR_UNSUPPORTED, "the voxel walk reads dense caches only");
     for (int i = 0; i < n_cams; ++i)
         if ((st = check_camera(&cams[i])) != FNR_OK) return st;
-    cudaError_t e = use_device(ctx->device);
+    cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_fail(e, "cudaSetDevice");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     MarchArgs a;

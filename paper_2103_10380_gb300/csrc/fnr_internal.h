@@ -128,11 +128,6 @@ private:
     bool pooled = false;
     cudaStream_t stream = nullptr;
 };
-// Make the device current, if it is not.
-inline cudaError_t use_device(int device) {
-    int cur = -1;
-    return cudaGetDevice(&cur) == cudaSuccess && cur == device ? cudaSuccess : cudaSetDevice(device);
-}
 // The armed cache-build fault (fnr_testing_mlp_fault), taken once: leaves the
 // arguments unchanged when none is armed.
 void take_mlp_fault(long long *wait_limit, long long *withhold);

@@ -234,7 +234,7 @@ extern "C" fnr_status fnr_render_mlp(fnr_context *ctx, const fnr_mlp *pos_mlp, c
     if ((st = make_render_const(params, &rc)) != FNR_OK) return st;
     if (rc.flags != 0u) return fail(FNR_ERR_UNSUPPORTED, "the uncached render takes no render flags");
     if ((st = check_camera(cam)) != FNR_OK) return st;
-    cudaError_t e = use_device(ctx->device);
+    cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_fail(e, "cudaSetDevice");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     FrameDesc F;
