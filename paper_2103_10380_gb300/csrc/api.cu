@@ -460,8 +460,16 @@ uint64_t fnr_cache_footprint(const fnr_cache_desc *d) {
     return layout_of(d).total;
 }
 
+// The dense stage of a brick build: its device memory, and the host tables it is being filled from. Copies from
+// pageable memory need not have read it when cudaMemcpyAsync returns (where the GPU reads the host's page tables they
+// are queued like any other), so the tables live until the stream has been waited for.
+struct DenseStage {
+    TempBuf mem;
+    std::vector<char> tables;
+};
+
 static fnr_status build_dense(fnr_context *ctx, const fnr_cache_desc *desc, const fnr_cache_source *src,
-                              bool records, TempBuf *stage, cudaStream_t s, fnr_cache **out);
+                              bool records, DenseStage *stage, cudaStream_t s, fnr_cache **out);
 
 // Dense cache -> FNR_LAYOUT_BRICKS cache: pool slots in brick-index order of
 // the occupied bricks, found on the GPU (only their count is read back, for the
@@ -555,10 +563,11 @@ fnr_status fnr_build_cache(fnr_context *ctx, const fnr_cache_desc *desc, const f
         dd.layout = FNR_LAYOUT_DENSE;
         const bool direct = src->kind == FNR_SRC_ARRAYS && src->location == FNR_LOC_DEVICE;
         fnr_cache *dense = nullptr;
-        TempBuf stage;
+        DenseStage stage;
         fnr_status st = build_dense(ctx, &dd, src, !direct, &stage, s, &dense);
         if (st != FNR_OK) return st;
         st = make_bricks(ctx, dense, layout_of(&dd, -1, !direct), direct ? src->uvw : nullptr, desc, s, out);
+        if (st != FNR_OK) cudaStreamSynchronize(s);  // what was queued has left the tables and the caller's arrays
         budget_uncharge(ctx, dense->footprint);
         delete dense;
         return st;
@@ -566,11 +575,11 @@ fnr_status fnr_build_cache(fnr_context *ctx, const fnr_cache_desc *desc, const f
     return build_dense(ctx, desc, src, true, nullptr, s, out);
 }
 
-
-// A dense cache, complete on return; or, with `stage`, the dense stage of a brick build in that buffer, complete in
-// the order of the stream (the caller deletes it and returns its charge, c->footprint).
+// A dense cache, complete on return; or, with `stage`, the dense stage of a brick build in that memory, complete in
+// the order of the stream (the caller keeps `stage` until then, deletes the cache and returns its charge,
+// c->footprint). On failure nothing that was queued is still running.
 static fnr_status build_dense(fnr_context *ctx, const fnr_cache_desc *desc, const fnr_cache_source *src,
-                              bool records, TempBuf *stage, cudaStream_t s, fnr_cache **out) {
+                              bool records, DenseStage *stage, cudaStream_t s, fnr_cache **out) {
     fnr_status st0;
     if (src->kind == FNR_SRC_MLP) {
         if ((st0 = check_mlp(src->pos_mlp, 1 + 3 * desc->D, "pos_mlp")) != FNR_OK) return st0;
@@ -596,8 +605,8 @@ static fnr_status build_dense(fnr_context *ctx, const fnr_cache_desc *desc, cons
     c->footprint = charge;
     c->ctx = ctx;
     if (stage) {
-        e = stage->alloc(ctx, L.total, s);
-        c->base = stage->p;
+        e = stage->mem.alloc(ctx, L.total, s);
+        c->base = stage->mem.p;
         c->owned = false;
     } else {
         e = dev_malloc(&c->base, L.total);
@@ -607,13 +616,13 @@ static fnr_status build_dense(fnr_context *ctx, const fnr_cache_desc *desc, cons
         delete c;
         return cuda_fail(e, "cache allocation");
     }
-    // The direction-bin tables and, where no build computes them, defined scales (1): adjacent sections, one upload
-    // (from pageable memory: the call returns when the buffer has been read).
+    // The direction-bin tables and, where no build computes them, defined scales (1): adjacent sections, one upload.
     std::vector<float> ct, qp;
     bin_tables(desc->l, ct, qp);
     const bool fp8 = desc->pos_precision == FNR_PREC_FP8_E4M3;
     const size_t n_ones = fp8 ? 0 : size_t(1 + 3 * desc->D);
-    std::vector<char> tables(size_t(L.off_scales - L.off_ct) + n_ones * 4, 0);
+    std::vector<char> own_tables, &tables = stage ? stage->tables : own_tables;
+    tables.assign(size_t(L.off_scales - L.off_ct) + n_ones * 4, 0);
     memcpy(tables.data(), ct.data(), ct.size() * 4);
     memcpy(tables.data() + (L.off_qp - L.off_ct), qp.data(), qp.size() * 4);
     const std::vector<float> ones(n_ones, 1.0f);
@@ -650,6 +659,7 @@ static fnr_status build_dense(fnr_context *ctx, const fnr_cache_desc *desc, cons
         st = cuda_fail(e, "build sync");
     }
     if (st != FNR_OK) {
+        cudaStreamSynchronize(s);
         if (c->owned) cudaFree(c->base);
         budget_uncharge(ctx, charge);
         delete c;
