@@ -398,17 +398,6 @@ fnr_status fnr_context_create(int32_t device, uint64_t hbm_budget_bytes, fnr_con
     ctx->device = device;
     ctx->budget = hbm_budget_bytes;
     cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device);
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = device;
-    uint64_t keep = kPoolKeepBytes;
-    if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess) {
-        ctx->pool = nullptr;
-        cudaGetLastError();
-    } else if (cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-        cudaGetLastError();
-    }
     *out = ctx;
     return FNR_OK;
 }
@@ -430,10 +419,7 @@ fnr_status fnr_context_destroy(fnr_context *ctx) {
         if (c->owned && c->base) cudaFree(c->base);
         delete c;
     }
-    if (ctx->pool) {
-        cudaDeviceSynchronize();  // temporaries are freed in stream order
-        cudaMemPoolDestroy(ctx->pool);
-    }
+    if (ctx->pool) cudaMemPoolDestroy(ctx->pool);  // its memory goes once every temporary's stream has freed it
     delete ctx;
     return FNR_OK;
 }

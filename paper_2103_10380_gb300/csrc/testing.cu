@@ -35,10 +35,25 @@ cudaError_t dev_malloc(void **p, size_t bytes) {
     return injected_failure() ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
 }
 
-cudaError_t TempBuf::alloc(const fnr_context *ctx, size_t bytes, cudaStream_t s) {
+static void make_pool(fnr_context *ctx) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = ctx->device;
+    uint64_t keep = kPoolKeepBytes;
+    if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess) {
+        ctx->pool = nullptr;
+        cudaGetLastError();
+    } else if (cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+    }
+}
+
+cudaError_t TempBuf::alloc(fnr_context *ctx, size_t bytes, cudaStream_t s) {
     release();
     if (injected_failure()) return cudaErrorMemoryAllocation;
-    pooled = ctx->pool && bytes <= kPooledBytes;
+    if (bytes <= kPooledBytes) std::call_once(ctx->pool_once, make_pool, ctx);
+    pooled = bytes <= kPooledBytes && ctx->pool;
     stream = s;
     const cudaError_t e = pooled ? cudaMallocFromPoolAsync(&p, bytes, ctx->pool, s) : cudaMalloc(&p, bytes);
     if (e != cudaSuccess) p = nullptr;
