@@ -200,6 +200,7 @@ public:
     ~PointsMlp();
     fnr_status prepare(fnr_context *ctx, const fnr_mlp *m, int out_stride, bool relu0, cudaStream_t s);
     fnr_status launch(const float *points, long long max_n, const unsigned long long *n_dev, float *out, cudaStream_t s);
+    const int *error_word() const;  // on the device, after prepare(): 0 unless a launch has failed
     fnr_status finish(cudaStream_t s);
 
 private:

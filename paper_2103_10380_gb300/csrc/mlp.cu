@@ -762,6 +762,8 @@ fnr_status PointsMlp::launch(const float *points, long long max_n, const unsigne
     return mlp_launch(A, impl->B.num_sms, s);
 }
 
+const int *PointsMlp::error_word() const { return impl->A.err; }
+
 fnr_status PointsMlp::finish(cudaStream_t s) { return mlp_finish(impl->A, s); }
 
 }  // namespace fnr
