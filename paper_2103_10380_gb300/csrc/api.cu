@@ -398,6 +398,7 @@ fnr_status fnr_context_create(int32_t device, uint64_t hbm_budget_bytes, fnr_con
     ctx->device = device;
     ctx->budget = hbm_budget_bytes;
     cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device);
+    ctx->pool = make_temp_pool(device);
     *out = ctx;
     return FNR_OK;
 }
@@ -419,7 +420,7 @@ fnr_status fnr_context_destroy(fnr_context *ctx) {
         if (c->owned && c->base) cudaFree(c->base);
         delete c;
     }
-    if (ctx->pool) cudaMemPoolDestroy(ctx->pool);  // its memory goes once every temporary's stream has freed it
+    destroy_temp_pool(ctx->pool);
     delete ctx;
     return FNR_OK;
 }

@@ -111,9 +111,8 @@ cudaError_t dev_malloc(T **p, size_t bytes) {
 // A temporary of one call, freed with the object in the order of stream `s`. Up to kPooledBytes it comes from the
 // context's pool of stream-ordered memory (a cudaMalloc and cudaFree pair takes 60 us, a small build had seven);
 // larger ones are allocated and freed (from a pool that does not keep them they cost twice as much). The pool
-// belongs to one context, is made by the first call that needs it (contexts may be made and destroyed while some
-// stream is captured), keeps at most kPoolKeepBytes between calls and is given back with the context; streams and
-// threads may share it.
+// belongs to one context, keeps at most kPoolKeepBytes between calls and is given back with the context; streams
+// and threads may share it.
 constexpr size_t kPooledBytes = size_t(64) << 20, kPoolKeepBytes = size_t(128) << 20;
 class TempBuf {
 public:
@@ -122,13 +121,17 @@ public:
     TempBuf(const TempBuf &) = delete;
     TempBuf &operator=(const TempBuf &) = delete;
     ~TempBuf() { release(); }
-    cudaError_t alloc(fnr_context *ctx, size_t bytes, cudaStream_t s);
+    cudaError_t alloc(const fnr_context *ctx, size_t bytes, cudaStream_t s);
     void release();
 
 private:
     bool pooled = false;
     cudaStream_t stream = nullptr;
 };
+// A context's pool, made with the context (40 us that its first build would pay otherwise; null if the device has
+// no such pools) and destroyed with it, without a wait: its memory goes when the last temporary's stream has freed it.
+cudaMemPool_t make_temp_pool(int device);
+void destroy_temp_pool(cudaMemPool_t pool);
 // The armed cache-build fault (fnr_testing_mlp_fault), taken once: leaves the
 // arguments unchanged when none is armed.
 void take_mlp_fault(long long *wait_limit, long long *withhold);
@@ -198,7 +201,7 @@ fnr_status check_mlp(const fnr_mlp *m, int n_out_min, const char *name);
 class PointsMlp {
 public:
     ~PointsMlp();
-    fnr_status prepare(fnr_context *ctx, const fnr_mlp *m, int out_stride, bool relu0, cudaStream_t s);
+    fnr_status prepare(const fnr_context *ctx, const fnr_mlp *m, int out_stride, bool relu0, cudaStream_t s);
     fnr_status launch(const float *points, long long max_n, const unsigned long long *n_dev, float *out, cudaStream_t s);
     const int *error_word() const;  // on the device, after prepare(): 0 unless a launch has failed
     fnr_status finish(cudaStream_t s);
@@ -210,7 +213,7 @@ private:
 class GridMlp {
 public:
     ~GridMlp();
-    fnr_status launch(fnr_context *ctx, const fnr_mlp *m, int mode, const fnr_cache_desc &d, const CacheView &v,
+    fnr_status launch(const fnr_context *ctx, const fnr_mlp *m, int mode, const fnr_cache_desc &d, const CacheView &v,
                       cudaStream_t s);
     fnr_status finish(cudaStream_t s);
 
@@ -241,6 +244,5 @@ struct fnr_context {
     std::set<fnr_cache *> caches;
     std::mutex serve_mu;
     fnr::Server *server = nullptr;
-    std::once_flag pool_once;
-    cudaMemPool_t pool = nullptr;  // temporaries (TempBuf); null before the first, or if the device has no such pools
+    cudaMemPool_t pool = nullptr;  // temporaries (TempBuf); null if the device has no such pools
 };

@@ -631,7 +631,7 @@ struct MlpBuffers {
 };
 
 // Lay out the weights and biases of m and fill the layer table of A (A.mode and its outputs per point are set).
-fnr_status mlp_prepare(fnr_context *ctx, const fnr_mlp *m, MlpArgs &A, MlpBuffers &B, cudaStream_t s) {
+fnr_status mlp_prepare(const fnr_context *ctx, const fnr_mlp *m, MlpArgs &A, MlpBuffers &B, cudaStream_t s) {
     B.num_sms = ctx->num_sms;
     size_t welems = 0, belems = 0;
     for (int i = 0; i < m->n_layers; ++i) {
@@ -710,7 +710,7 @@ struct GridMlp::Impl {
 
 GridMlp::~GridMlp() { delete impl; }
 
-fnr_status GridMlp::launch(fnr_context *ctx, const fnr_mlp *m, int mode, const fnr_cache_desc &d,
+fnr_status GridMlp::launch(const fnr_context *ctx, const fnr_mlp *m, int mode, const fnr_cache_desc &d,
                            const CacheView &v, cudaStream_t s) {
     impl = new Impl();
     MlpArgs &A = impl->A;
@@ -743,7 +743,7 @@ struct PointsMlp::Impl {
 
 PointsMlp::~PointsMlp() { delete impl; }
 
-fnr_status PointsMlp::prepare(fnr_context *ctx, const fnr_mlp *m, int out_stride, bool relu0, cudaStream_t s) {
+fnr_status PointsMlp::prepare(const fnr_context *ctx, const fnr_mlp *m, int out_stride, bool relu0, cudaStream_t s) {
     impl = new Impl();
     memset(&impl->A, 0, sizeof(impl->A));
     impl->A.mode = 2;

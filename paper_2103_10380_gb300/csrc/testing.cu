@@ -35,25 +35,38 @@ cudaError_t dev_malloc(void **p, size_t bytes) {
     return injected_failure() ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
 }
 
-static void make_pool(fnr_context *ctx) {
+// A stream capture, in whichever thread, does not mind these calls of this thread: pools have no stream.
+struct OutsideCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    OutsideCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~OutsideCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+cudaMemPool_t make_temp_pool(int device) {
+    OutsideCapture relaxed;
     cudaMemPoolProps props = {};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = ctx->device;
+    props.location.id = device;
     uint64_t keep = kPoolKeepBytes;
-    if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess) {
-        ctx->pool = nullptr;
+    cudaMemPool_t pool = nullptr;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
         cudaGetLastError();
-    } else if (cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-        cudaGetLastError();
+        return nullptr;
     }
+    if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
+    return pool;
 }
 
-cudaError_t TempBuf::alloc(fnr_context *ctx, size_t bytes, cudaStream_t s) {
+void destroy_temp_pool(cudaMemPool_t pool) {
+    OutsideCapture relaxed;
+    if (pool) cudaMemPoolDestroy(pool);
+}
+
+cudaError_t TempBuf::alloc(const fnr_context *ctx, size_t bytes, cudaStream_t s) {
     release();
     if (injected_failure()) return cudaErrorMemoryAllocation;
-    if (bytes <= kPooledBytes) std::call_once(ctx->pool_once, make_pool, ctx);
-    pooled = bytes <= kPooledBytes && ctx->pool;
+    pooled = ctx->pool && bytes <= kPooledBytes;
     stream = s;
     const cudaError_t e = pooled ? cudaMallocFromPoolAsync(&p, bytes, ctx->pool, s) : cudaMalloc(&p, bytes);
     if (e != cudaSuccess) p = nullptr;
