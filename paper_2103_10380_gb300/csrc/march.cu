@@ -14,8 +14,9 @@
 //   a9 RGBA (+ optional per-ray counters and per-sample cells)
 //
 // The kernels for FNR_RENDER_SKIP_EMPTY (density loads only in occupied
-// bricks) and for FNR_LAYOUT_BRICKS caches are the same template with SKIP
-// (and BRICKS) set, compiled in march_skip.cu / march_bricks.cu so the kernel
+// bricks), for FNR_LAYOUT_BRICKS caches and for renders that write every
+// sample's cell are the same template with SKIP (and BRICKS), CELLS set,
+// compiled in march_skip.cu, march_bricks.cu and march_*cells.cu so the kernel
 // sets build in parallel.
 #include "march_device.cuh"
 
@@ -25,8 +26,8 @@ namespace {
 
 using namespace dev;
 
-template <int PREC, int D, bool SKIP, bool BRICKS>
-__global__ void __launch_bounds__(FNR_BLOCK, dev::min_blocks<PREC, D>())
+template <int PREC, int D, bool SKIP, bool BRICKS, bool CELLS>
+__global__ void __launch_bounds__(FNR_BLOCK, dev::min_blocks<PREC, D, SKIP, CELLS>())
     march_kernel(const __grid_constant__ MarchArgs A) {
     allow_next_grid();  // the next render launch may be scheduled as SMs free up
     const int tile = static_cast<int>((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
@@ -39,11 +40,12 @@ __global__ void __launch_bounds__(FNR_BLOCK, dev::min_blocks<PREC, D>())
     tile_origin(F, t, x0, y0);
     const int lane = threadIdx.x & 31;
     const int px = x0 + (lane & (kTileW - 1)), py = y0 + lane / kTileW;
-    __shared__ QueueFor<PREC, D, BRICKS> queues[FNR_BLOCK / 32];
-    march_tile_queued<PREC, D, SKIP, BRICKS>(A.c, A.r, F, px, py, px < F.W && py < F.H, queues[threadIdx.x >> 5]);
+    __shared__ QueueFor<PREC, D, BRICKS, CELLS> queues[FNR_BLOCK / 32];
+    march_tile_queued<PREC, D, SKIP, BRICKS, CELLS>(A.c, A.r, F, px, py, px < F.W && py < F.H,
+                                                    queues[threadIdx.x >> 5]);
 }
 
-template <int PREC, int D, bool SKIP, bool BRICKS>
+template <int PREC, int D, bool SKIP, bool BRICKS, bool CELLS>
 cudaError_t launch_t(const MarchArgs &a, cudaStream_t s) {
     const int threads = FNR_BLOCK;
     const int warps_per_block = threads / 32;
@@ -60,60 +62,63 @@ cudaError_t launch_t(const MarchArgs &a, cudaStream_t s) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, march_kernel<PREC, D, SKIP, BRICKS>, a);
+    return cudaLaunchKernelEx(&cfg, march_kernel<PREC, D, SKIP, BRICKS, CELLS>, a);
 }
 
-template <int PREC, bool SKIP, bool BRICKS>
+template <int PREC, bool SKIP, bool BRICKS, bool CELLS>
 cudaError_t launch_p(const MarchArgs &a, cudaStream_t s) {
 #ifdef FNR_TUNING_D8_ONLY  // faster builds for launch-shape sweeps: D = 8 only
-    return a.c.D == 8 ? launch_t<PREC, 8, SKIP, BRICKS>(a, s) : cudaErrorInvalidValue;
+    return a.c.D == 8 ? launch_t<PREC, 8, SKIP, BRICKS, CELLS>(a, s) : cudaErrorInvalidValue;
 #endif
     switch (a.c.D) {
-        case 1: return launch_t<PREC, 1, SKIP, BRICKS>(a, s);
-        case 2: return launch_t<PREC, 2, SKIP, BRICKS>(a, s);
-        case 3: return launch_t<PREC, 3, SKIP, BRICKS>(a, s);
-        case 4: return launch_t<PREC, 4, SKIP, BRICKS>(a, s);
-        case 5: return launch_t<PREC, 5, SKIP, BRICKS>(a, s);
-        case 6: return launch_t<PREC, 6, SKIP, BRICKS>(a, s);
-        case 7: return launch_t<PREC, 7, SKIP, BRICKS>(a, s);
-        case 8: return launch_t<PREC, 8, SKIP, BRICKS>(a, s);
-        case 9: return launch_t<PREC, 9, SKIP, BRICKS>(a, s);
-        case 10: return launch_t<PREC, 10, SKIP, BRICKS>(a, s);
-        case 11: return launch_t<PREC, 11, SKIP, BRICKS>(a, s);
-        case 12: return launch_t<PREC, 12, SKIP, BRICKS>(a, s);
-        case 13: return launch_t<PREC, 13, SKIP, BRICKS>(a, s);
-        case 14: return launch_t<PREC, 14, SKIP, BRICKS>(a, s);
-        case 15: return launch_t<PREC, 15, SKIP, BRICKS>(a, s);
-        case 16: return launch_t<PREC, 16, SKIP, BRICKS>(a, s);
+        case 1: return launch_t<PREC, 1, SKIP, BRICKS, CELLS>(a, s);
+        case 2: return launch_t<PREC, 2, SKIP, BRICKS, CELLS>(a, s);
+        case 3: return launch_t<PREC, 3, SKIP, BRICKS, CELLS>(a, s);
+        case 4: return launch_t<PREC, 4, SKIP, BRICKS, CELLS>(a, s);
+        case 5: return launch_t<PREC, 5, SKIP, BRICKS, CELLS>(a, s);
+        case 6: return launch_t<PREC, 6, SKIP, BRICKS, CELLS>(a, s);
+        case 7: return launch_t<PREC, 7, SKIP, BRICKS, CELLS>(a, s);
+        case 8: return launch_t<PREC, 8, SKIP, BRICKS, CELLS>(a, s);
+        case 9: return launch_t<PREC, 9, SKIP, BRICKS, CELLS>(a, s);
+        case 10: return launch_t<PREC, 10, SKIP, BRICKS, CELLS>(a, s);
+        case 11: return launch_t<PREC, 11, SKIP, BRICKS, CELLS>(a, s);
+        case 12: return launch_t<PREC, 12, SKIP, BRICKS, CELLS>(a, s);
+        case 13: return launch_t<PREC, 13, SKIP, BRICKS, CELLS>(a, s);
+        case 14: return launch_t<PREC, 14, SKIP, BRICKS, CELLS>(a, s);
+        case 15: return launch_t<PREC, 15, SKIP, BRICKS, CELLS>(a, s);
+        case 16: return launch_t<PREC, 16, SKIP, BRICKS, CELLS>(a, s);
         default: return cudaErrorInvalidValue;
     }
 }
 
-template <bool SKIP, bool BRICKS>
+template <bool SKIP, bool BRICKS, bool CELLS>
 cudaError_t launch_all(const MarchArgs &a, cudaStream_t s) {
     switch (a.c.pos_prec) {
-        case FNR_PREC_FP32: return launch_p<FNR_PREC_FP32, SKIP, BRICKS>(a, s);
-        case FNR_PREC_FP16: return launch_p<FNR_PREC_FP16, SKIP, BRICKS>(a, s);
-        case FNR_PREC_FP8_E4M3: return launch_p<FNR_PREC_FP8_E4M3, SKIP, BRICKS>(a, s);
+        case FNR_PREC_FP32: return launch_p<FNR_PREC_FP32, SKIP, BRICKS, CELLS>(a, s);
+        case FNR_PREC_FP16: return launch_p<FNR_PREC_FP16, SKIP, BRICKS, CELLS>(a, s);
+        case FNR_PREC_FP8_E4M3: return launch_p<FNR_PREC_FP8_E4M3, SKIP, BRICKS, CELLS>(a, s);
         default: return cudaErrorInvalidValue;
     }
 }
 
 }  // namespace
 
-#if defined(FNR_MARCH_SKIP_UNIT)
-cudaError_t launch_march_skip(const MarchArgs &a, cudaStream_t s) { return launch_all<true, false>(a, s); }
-#elif defined(FNR_MARCH_BRICKS_UNIT)
-cudaError_t launch_march_bricks(const MarchArgs &a, cudaStream_t s) { return launch_all<true, true>(a, s); }
+#if defined(FNR_MARCH_LAUNCHER)  // one of the other units: its launcher's name and SKIP, BRICKS, CELLS
+cudaError_t FNR_MARCH_LAUNCHER(const MarchArgs &a, cudaStream_t s) { return launch_all<FNR_MARCH_FORM>(a, s); }
 #else
-cudaError_t launch_march_skip(const MarchArgs &a, cudaStream_t s);    // march_skip.cu
-cudaError_t launch_march_bricks(const MarchArgs &a, cudaStream_t s);  // march_bricks.cu
+cudaError_t launch_march_skip(const MarchArgs &a, cudaStream_t s);          // march_skip.cu
+cudaError_t launch_march_bricks(const MarchArgs &a, cudaStream_t s);        // march_bricks.cu
+cudaError_t launch_march_cells(const MarchArgs &a, cudaStream_t s);         // march_cells.cu
+cudaError_t launch_march_skip_cells(const MarchArgs &a, cudaStream_t s);    // march_skip_cells.cu
+cudaError_t launch_march_bricks_cells(const MarchArgs &a, cudaStream_t s);  // march_bricks_cells.cu
 
 cudaError_t launch_march(const MarchArgs &a, cudaStream_t s) {
     if (a.total_tiles <= 0) return cudaSuccess;
-    if (a.c.layout == FNR_LAYOUT_BRICKS) return launch_march_bricks(a, s);  // always skipping
-    if (a.r.flags & FNR_RENDER_SKIP_EMPTY) return launch_march_skip(a, s);
-    return launch_all<false, false>(a, s);
+    const bool cells = a.f[0].cells != nullptr;                   // of every view of a launch or of none
+    if (a.c.layout == FNR_LAYOUT_BRICKS)                          // always skipping
+        return cells ? launch_march_bricks_cells(a, s) : launch_march_bricks(a, s);
+    if (a.r.flags & FNR_RENDER_SKIP_EMPTY) return cells ? launch_march_skip_cells(a, s) : launch_march_skip(a, s);
+    return cells ? launch_march_cells(a, s) : launch_all<false, false, false>(a, s);
 }
 #endif
 

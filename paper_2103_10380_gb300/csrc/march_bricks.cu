@@ -2,5 +2,6 @@
 // (densities and records in brick pools behind a page table; empty bricks
 // skipped): march.cu's template instantiated with SKIP = BRICKS = true in a
 // translation unit of its own, so the kernel sets compile in parallel.
-#define FNR_MARCH_BRICKS_UNIT
+#define FNR_MARCH_LAUNCHER launch_march_bricks
+#define FNR_MARCH_FORM true, true, false
 #include "march.cu"

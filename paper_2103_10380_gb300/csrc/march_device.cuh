@@ -6,6 +6,8 @@
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
 
+#include <type_traits>
+
 #include "fnr_internal.h"
 
 namespace fnr {
@@ -33,13 +35,22 @@ namespace dev {
 // 78.0 / 80.2 (4). E4M3 carries offsets and scales besides and spills at 9 blocks (110). Longer records need their
 // registers: FP32 at 7 / 8 / 9 blocks 101.6 / 94.8 / 99.4 (D = 12) and 118.8 / 115.6 / 118.0 (16); E4M3, D = 12, groups
 // of 6 at 7 blocks 99.5, of 5 at 8 116.8; D = 16, groups of 6 at 6 / 7 blocks 126 / 130.
-template <int PREC, int D, bool BRICKS>
+//
+// CELLS, renders that write every sample's cell: groups of 8, whose stores fill a lane's 32-byte sectors (N cells a ray
+// are most of what is moved), and fewer blocks. 200 x 200 / 640 x 640, k = 256, N = 128, D = 8, cells written by the
+// kernels above -> here, in us: FP32 123.7 -> 101.8 / 329 -> 318, with skipping 95.8 -> 66.6 / 322 -> 287, bricks 94.5 ->
+// 84.6 / 326 -> 317; E4M3 107.5 -> 75.3 / 307 -> 286. 5 / 6 / 7 / 8 blocks: FP32 with skipping 66.6 / 78.9 / 85.8 / 98.4,
+// E4M3 75.3 / 87.7 / 99.1 / 115.2, level at most where they are not ahead; but FP16 without skipping, whose kernels need
+// no more registers, 322.5 at 5 and 317.6 at 8 (640 x 640).
+template <int PREC, int D, bool BRICKS, bool CELLS>
 __host__ __device__ constexpr int group_size() {
+    if (CELLS) return 8;
     if (PREC == FNR_PREC_FP8_E4M3) return D <= 8 ? 5 : 6;
     return D <= 6 && !BRICKS ? 6 : 5;
 }
-template <int PREC, int D>
+template <int PREC, int D, bool SKIP = false, bool CELLS = false>
 __host__ __device__ constexpr int min_blocks() {
+    if (CELLS) return PREC == FNR_PREC_FP16 && D <= 8 && !SKIP ? 8 : 5;
     if (PREC == FNR_PREC_FP8_E4M3) return D <= 8 ? 8 : (D <= 12 ? 7 : 6);
     return PREC == FNR_PREC_FP32 && D > 8 ? 8 : 9;
 }
@@ -590,8 +601,8 @@ struct WarpQueue {
     int obr[OFFS ? kQCap : 1];  // offset brick of each entry
     float sc[OFFS ? 3 * D : 1]; // scale of (u, v, w) channel ch D + j
 };
-template <int PREC, int D, bool BRICKS = false>
-using QueueFor = WarpQueue<D, PREC == FNR_PREC_FP8_E4M3, queue_cap(group_size<PREC, D, BRICKS>())>;
+template <int PREC, int D, bool BRICKS = false, bool CELLS = false>
+using QueueFor = WarpQueue<D, PREC == FNR_PREC_FP8_E4M3, queue_cap(group_size<PREC, D, BRICKS, CELLS>())>;
 
 // SKIP (FNR_RENDER_SKIP_EMPTY): a sample in a brick without stored density is
 // known to be empty, so only samples in occupied bricks load their density; the
@@ -599,10 +610,12 @@ using QueueFor = WarpQueue<D, PREC == FNR_PREC_FP8_E4M3, queue_cap(group_size<PR
 // BRICKS (FNR_LAYOUT_BRICKS, implies SKIP): densities and records live in brick
 // pools in brick-index order; an occupied sample's pool slot is the brick's rank
 // among the occupied bricks, and the queue carries pool indices instead of cells.
-template <int PREC, int D, bool SKIP, bool BRICKS = false>
+// CELLS: every sample's cell is written to F.cells (null in all other instantiations).
+template <int PREC, int D, bool SKIP, bool BRICKS = false, bool CELLS = false>
 __device__ __forceinline__ void march_tile_queued(const CacheView &c, const RenderConst &r, const FrameDesc &F,
-                                                  int px, int py, bool active, QueueFor<PREC, D, BRICKS> &q) {
-    constexpr int kUnroll = group_size<PREC, D, BRICKS>();
+                                                  int px, int py, bool active,
+                                                  QueueFor<PREC, D, BRICKS, CELLS> &q) {
+    constexpr int kUnroll = group_size<PREC, D, BRICKS, CELLS>();
     constexpr bool kOffs = PREC == FNR_PREC_FP8_E4M3;
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -624,9 +637,14 @@ __device__ __forceinline__ void march_tile_queued(const CacheView &c, const Rend
     unsigned long long S = 0;
     const unsigned long long s_thr = static_cast<unsigned long long>(r.s_thr);
     int n_look = 0, n_occ = 0, n_steps = r.N;
-    const long long pix = active ? static_cast<long long>(py) * F.W + px : 0;
-    int32_t *cells_out = (active && F.cells) ? F.cells + pix * r.N : nullptr;
-    if (F.cells) wait_prior_grid();  // per-sample cells are written while marching
+    // The lane's pixel, -1 without one, in one register through the whole march (found again from px and py at the end
+    // it took one more, which FP32 spills: 88.8 us, here 87.7, 800 x 800 as above). The kernels that write cells have
+    // use for all 64 bits from the start.
+    using Pixel = std::conditional_t<CELLS, long long, int>;
+    Pixel pix = active ? static_cast<Pixel>(py) * F.W + px : -1;
+    if constexpr (!CELLS) asm volatile("" : "+r"(pix));
+    int32_t *cells_out = (CELLS && active) ? F.cells + static_cast<long long>(pix) * r.N : nullptr;
+    if (CELLS) wait_prior_grid();  // per-sample cells are written while marching
     bool done = !active;
     if (cells_out)
         for (int i = 0; i < R.i_lo; ++i) cells_out[i] = -1;
@@ -678,11 +696,11 @@ __device__ __forceinline__ void march_tile_queued(const CacheView &c, const Rend
     // empty-group test by the maximum density (measured faster for binary32 densities only)
     constexpr bool kMaxTest = PREC == FNR_PREC_FP32;
     // skipping passes over runs of samples in empty space (not when every sample's cell is written)
-    const bool jump = SKIP && F.cells == nullptr;
+    constexpr bool kJump = SKIP && !CELLS;
     int qn = 0;
     for (int i0 = lo_w; i0 < hi_w; i0 += kUnroll) {
         if (!__any_sync(FULL, !done)) break;
-        if (SKIP && jump) {
+        if constexpr (kJump) {
             // The warp moves on, a step at a time, to the first sample some marching lane must
             // still test; each step is one cube of empty jump bricks for every lane, and the
             // steps stop as soon as one lane cannot advance.
@@ -901,7 +919,7 @@ __device__ __forceinline__ void march_tile_queued(const CacheView &c, const Rend
         flush(0, qn);
     }
     wait_prior_grid();
-    if (!active) return;
+    if (pix < 0) return;
     if (cells_out) {
         if (done)
             for (int i = n_steps; i < r.N; ++i) cells_out[i] = -2;

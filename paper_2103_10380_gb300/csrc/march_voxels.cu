@@ -6,12 +6,10 @@ namespace fnr {
 
 cudaError_t launch_march_voxels(const MarchArgs &a, cudaStream_t s) {
     if (a.total_tiles <= 0) return cudaSuccess;
-    if ((a.r.flags & FNR_RENDER_SKIP_EMPTY) == 0u) return launch_voxels_prec<kVoxPlain>(a, s);
-    // the passes over empty cubes need the distance field and a walk that records no cells
-    bool jump = a.c.dist != nullptr;
-    for (int f = 0; f < a.n_frames; ++f)
-        if (a.f[f].cells) jump = false;
-    return jump ? launch_march_voxels_jump(a, s) : launch_march_voxels_skip(a, s);
+    const bool skip = (a.r.flags & FNR_RENDER_SKIP_EMPTY) != 0u;
+    if (a.f[0].cells != nullptr)  // of every view of a launch or of none
+        return skip ? launch_march_voxels_skip_cells(a, s) : launch_march_voxels_cells(a, s);
+    return skip ? launch_march_voxels_jump(a, s) : launch_voxels_prec<kVoxPlain>(a, s);
 }
 
 }  // namespace fnr

@@ -19,12 +19,12 @@
 // t_far in r.dt (the walk has no sample spacing) and r.s_thr is the threshold
 // on sum floor(fp32(sigma delta) 2^32).
 //
-// The kernel is instantiated three times per (precision, D), one form per
+// The kernel is instantiated four times per (precision, D), one form per
 // translation unit: the plain walk (march_voxels.cu), the walk that skips the
-// density loads of empty bricks (march_voxels_skip.cu), and the same with the
-// one-step passes over empty cubes, used when no per-cell output is asked for
-// (march_voxels_jump.cu). Each form carries only its own code: the brick
-// arithmetic alone cost the plain walk 10%.
+// density loads of empty bricks and passes over empty cubes in one step
+// (march_voxels_jump.cu), and both without the passes when every walked cell is
+// written (march_voxels_cells.cu, march_voxels_skip_cells.cu). Each form carries
+// only its own code: the brick arithmetic alone cost the plain walk 10%.
 #pragma once
 #include <type_traits>
 
@@ -32,7 +32,7 @@
 
 namespace fnr {
 
-enum VoxelForm { kVoxPlain = 0, kVoxSkip = 1, kVoxJump = 2 };
+enum VoxelForm { kVoxPlain = 0, kVoxJump = 1, kVoxCells = 2, kVoxSkipCells = 3 };
 
 namespace {
 
@@ -42,16 +42,24 @@ using namespace dev;
 // over an empty cube per group: at 8 the skipping kernel stalled on instruction fetch (2.6 of 9.6 cycles an
 // instruction) and walked up to 7 cells into empty space. 800 x 800, k = 512, 8 / 6 / 4 / 3 / 2 cells: FP32 with
 // skipping 876 / 766 / 642 / 652 / 688 us, E4M3 1487 / 1233 / 885 / 776 / 795; FP32 plain 1064 / - / 1002.
+// The forms that write every walked cell are bound by those stores, 4 bytes a cell at 3k cells a ray: eight at a time
+// fill a lane's 32-byte sectors, and few blocks leave them in L2 until they are full. With skipping, 640 x 640, k = 128,
+// FP32: 4 / 6 / 8 cells at 4 blocks 896 / 912 / 798 us, 8 cells at 4 / 5 / 6 / 7 blocks 798 / 814 / 855 / 850. Groups and
+// blocks as the other forms' -> these, 640 x 640, k = 128 and 256 x 256, k = 192: FP32 956 -> 856 and 415 -> 299, with
+// skipping 952 -> 798 and 423 -> 256; E4M3 971 -> 818 and 431 -> 254, with skipping 962 -> 793 and 451 -> 263; FP16 967 ->
+// 852, with skipping 966 -> 814.
 template <int PREC, int FORM>
 constexpr int walk_group() {
+    if (FORM == kVoxCells || FORM == kVoxSkipCells) return 8;
     return PREC == FNR_PREC_FP8_E4M3 && FORM == kVoxJump ? 3 : 4;
 }
 
 // Minimum resident blocks per SM (registers against latency). FP32 with / without skipping at 6 / 7 / 8 blocks:
 // 640 / 613 / 581 and 994 / 932 / 886 us; FP16 without skipping (512 x 512, k = 256) 181 / 171 / 177; E4M3 with it
 // 720 / 719 / 704.
-template <int PREC>
+template <int PREC, int FORM>
 constexpr int walk_blocks() {
+    if (FORM == kVoxCells || FORM == kVoxSkipCells) return 4;
     return PREC == FNR_PREC_FP16 ? 7 : 8;
 }
 
@@ -260,7 +268,7 @@ struct VoxelWalk {
 };
 
 template <int PREC, int D, int FORM>
-__global__ void __launch_bounds__(FNR_BLOCK, walk_blocks<PREC>())
+__global__ void __launch_bounds__(FNR_BLOCK, walk_blocks<PREC, FORM>())
     march_voxels_kernel(const __grid_constant__ MarchArgs A) {
     allow_next_grid();
     constexpr unsigned FULL = 0xffffffffu;
@@ -306,17 +314,18 @@ __global__ void __launch_bounds__(FNR_BLOCK, walk_blocks<PREC>())
         dd[1] = __fdiv_rn(wy, len);
         dd[2] = __fdiv_rn(wz, len);
     }
-    const bool skip = FORM != kVoxPlain && (r.flags & FNR_RENDER_SKIP_EMPTY) != 0u;
+    constexpr bool kCells = FORM == kVoxCells || FORM == kVoxSkipCells;
+    constexpr bool kSkip = FORM == kVoxJump || FORM == kVoxSkipCells;
     // Skipping without per-cell output also passes over whole empty cubes of jump
     // bricks in one step (VoxelWalk::pass_cube), from the cache's distance field.
-    const bool jumps = FORM == kVoxJump && skip && F.cells == nullptr && c.dist != nullptr;
+    constexpr bool kJump = FORM == kVoxJump;
     float T = 1.0f, Cr = 0.0f, Cg = 0.0f, Cb = 0.0f;
     unsigned long long S = 0;
     int n_gen = 0, n_steps = 0, n_look = 0, n_occ = 0;
     bool term = false;
     const long long pix = active ? static_cast<long long>(py) * F.W + px : 0;
-    int32_t *cells_out = (active && F.cells) ? F.cells + pix * r.N : nullptr;
-    if (F.cells) wait_prior_grid();  // cells are written while walking
+    int32_t *cells_out = (kCells && active) ? F.cells + pix * r.N : nullptr;
+    if (kCells) wait_prior_grid();  // cells are written while walking
 
     auto walk = [&](auto recip) {
         VoxelWalk<decltype(recip)::value> Wk;
@@ -333,7 +342,7 @@ __global__ void __launch_bounds__(FNR_BLOCK, walk_blocks<PREC>())
                 brick[u] = 0;
                 obr[u] = 0;
                 dl[u] = 0.0f;
-                if (jumps && u == 0 && Wk.live && !term && n_gen < r.N) {
+                if (kJump && u == 0 && Wk.live && !term && n_gen < r.N) {
                     // One pass per group (more per group measured slower: each costs a dozen exact divisions
                     // and the lanes of a warp take different ones). d > 0: the jump bricks within Chebyshev
                     // distance d - 1 of the current one are empty.
@@ -359,11 +368,15 @@ __global__ void __launch_bounds__(FNR_BLOCK, walk_blocks<PREC>())
                     ++n_gen;
                 }
             }
+            // The cell indices as they are: rebuilt from the walk's coordinates where they are used, they kept more
+            // registers alive (FP32 plain 776 us, now 749; FP16 plain 174, now 168).
+#pragma unroll
+            for (int u = 0; u < kVU; ++u) asm volatile("" : "+r"(cell[u]));
 #pragma unroll
             for (int u = 0; u < kVU; ++u) {
                 sg[u] = 0.0f;
                 if (((gen >> u) & 1u) && dl[u] > 0.0f) {
-                    const bool load = !skip || brick_occupied(c, brick[u]) != 0u;
+                    const bool load = !kSkip || brick_occupied(c, brick[u]) != 0u;
                     if (load) {
                         sg[u] = load_sigma<PREC>(c, cell[u], R.sigma_scale);
                         looked |= 1u << u;
@@ -495,8 +508,9 @@ cudaError_t launch_voxels_prec(const MarchArgs &a, cudaStream_t s) {
 
 }  // namespace
 
-// The skipping forms of the walk (march_voxels_skip.cu, march_voxels_jump.cu).
-cudaError_t launch_march_voxels_skip(const MarchArgs &a, cudaStream_t s);
+// The other forms of the walk (march_voxels_jump.cu, march_voxels_cells.cu, march_voxels_skip_cells.cu).
 cudaError_t launch_march_voxels_jump(const MarchArgs &a, cudaStream_t s);
+cudaError_t launch_march_voxels_cells(const MarchArgs &a, cudaStream_t s);
+cudaError_t launch_march_voxels_skip_cells(const MarchArgs &a, cudaStream_t s);
 
 }  // namespace fnr

@@ -1,0 +1,12 @@
+// march_voxels_skip_cells.cu -- the voxel walk's instantiations that skip the
+// density loads of empty bricks and write every walked cell (march_voxels.cuh),
+// compiled apart from the others.
+#include "march_voxels.cuh"
+
+namespace fnr {
+
+cudaError_t launch_march_voxels_skip_cells(const MarchArgs &a, cudaStream_t s) {
+    return launch_voxels_prec<kVoxSkipCells>(a, s);
+}
+
+}  // namespace fnr
