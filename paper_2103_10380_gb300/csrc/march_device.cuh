@@ -33,8 +33,10 @@ namespace dev {
 // 87.7, with skipping 87.9 -> 78.4, bricks 100 -> 89; FP16 81.2 -> 78.1, 81.7 -> 76.6, bricks 103 -> 87; E4M3 94.8 ->
 // 91.7, 98.4 -> 90.6. 5 / 6 / 8 samples at 9 blocks, FP32: 87.7 / 90.0 / 93.4 (D = 8), 82.2 / 79.3 / 82.1 (6), 82.0 /
 // 78.0 / 80.2 (4). E4M3 carries offsets and scales besides and spills at 9 blocks (110). Longer records need their
-// registers: FP32 at 7 / 8 / 9 blocks 101.6 / 94.8 / 99.4 (D = 12) and 118.8 / 115.6 / 118.0 (16); E4M3, D = 12, groups
-// of 6 at 7 blocks 99.5, of 5 at 8 116.8; D = 16, groups of 6 at 6 / 7 blocks 126 / 130.
+// registers: FP32 at 7 / 8 / 9 blocks 101.6 / 94.8 / 99.4 (D = 12) and 118.8 / 115.6 / 118.0 (16). 800 x 800, k = 400,
+// groups of 6: E4M3 at 6 / 7 / 8 blocks 96.0 / 92.3 / 96.6 (D = 12), 101.5 / 97.2 / 101.0 (14), 110.2 / 100.2 / 116.2
+// (16). FP16, groups of 5 at 8 / 9 blocks: 79.1 / 75.2 (12), 79.5 / 76.1 (14), 83.9 / 87.7 (15, whose kernel spills 28
+// bytes at 9), 81.2 / 78.2 (16).
 //
 // CELLS, renders that write every sample's cell: groups of 8, whose stores fill a lane's 32-byte sectors (N cells a ray
 // are most of what is moved), and fewer blocks. 200 x 200 / 640 x 640, k = 256, N = 128, D = 8, cells written by the
@@ -51,8 +53,8 @@ __host__ __device__ constexpr int group_size() {
 template <int PREC, int D, bool SKIP = false, bool CELLS = false>
 __host__ __device__ constexpr int min_blocks() {
     if (CELLS) return PREC == FNR_PREC_FP16 && D <= 8 && !SKIP ? 8 : 5;
-    if (PREC == FNR_PREC_FP8_E4M3) return D <= 8 ? 8 : (D <= 12 ? 7 : 6);
-    return PREC == FNR_PREC_FP32 && D > 8 ? 8 : 9;
+    if (PREC == FNR_PREC_FP8_E4M3) return D <= 8 ? 8 : 7;
+    return (PREC == FNR_PREC_FP32 && D > 8) || (PREC == FNR_PREC_FP16 && D == 15) ? 8 : 9;
 }
 
 // Whether an occupied sample's record is prefetched into L2 when the sample is queued. E4M3 records (24 bytes) and
