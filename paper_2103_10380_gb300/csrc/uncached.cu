@@ -3,7 +3,8 @@
 // composited with Eq. 5 and Eq. 1 exactly as the cached march does.
 //
 //   directions_kernel: every ray's unit direction, and F_dir over them;
-//   then, batch by batch of rays (at most 8 Mi samples):
+//   then, batch by batch of rays (about 8 Mi samples, or 16 Ki rays if that
+//     is more):
 //   samples_kernel: the inside samples' positions in one compact list (a
 //     warp-aggregated atomic hands each ray its range);
 //   F_pos over the list (PointsMlp; its length stays on the device);
@@ -17,6 +18,9 @@
 // 128 samples has 9 GB of them in one piece, whose allocation and release and
 // whose wait for the number of samples took 5 of 45 ms. Batches of 2 / 4 / 8 Mi
 // samples: 44.0 / 40.6 / 39.0 ms (each launch has its ramp and its last wave).
+// Compositing is a thread per ray, so a batch also holds at least 16 Ki rays:
+// 256 x 256 x 4096 at 2 / 4 / 8 / 16 / 32 / 64 Ki rays 215 / 166 / 143 / 135 /
+// 134 / 139 ms. All batches are of one size but for the last.
 #include <algorithm>
 
 #include "march_device.cuh"
@@ -280,9 +284,10 @@ extern "C" fnr_status fnr_render_mlp(fnr_context *ctx, const fnr_mlp *pos_mlp, c
     if (!budget_charge(ctx, bytes))
         return fail(FNR_ERR_BUDGET, "the uncached render needs %llu bytes of temporaries",
                     (unsigned long long)bytes);
-    constexpr long long kBatchPoints = 1LL << 23;
-    const long long batch = std::min<long long>(n_rays, std::max<long long>(kBatchPoints / rc.N, 1));
-    const long long n_batches = (n_rays + batch - 1) / batch, batch_pts = batch * rc.N;
+    constexpr long long kBatchPoints = 1LL << 23, kBatchRays = 1LL << 14;
+    const long long most = std::max<long long>(kBatchPoints / rc.N, kBatchRays);
+    const long long n_batches = (n_rays + most - 1) / most, batch = (n_rays + n_batches - 1) / n_batches;
+    const long long batch_pts = batch * rc.N;
     const bool staged = n_batches > 1;
     TempBuf points, pos_out, dirs, dir_out, offset, totals, image;
     PointsMlp pos, dir;

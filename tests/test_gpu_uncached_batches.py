@@ -1,4 +1,4 @@
-"""The uncached render's batches of rays (at most 8 Mi samples, or 16 Ki rays, each).
+"""The uncached render's batches of rays (8 Mi samples each, or 16 Ki rays if that is more).
 
 A view of several batches equals, byte for byte, the same rays rendered as strips of one batch each: shifting the
 principal point by whole rows leaves (py + 1/2) - cy, and so every ray, the same binary32 number, and neither the
@@ -12,7 +12,7 @@ import scenegen
 
 pytestmark = pytest.mark.gpu
 
-N = 512
+N = 512  # 16 Ki rays are 8 Mi samples
 ONE, SEVERAL = (211, 38), (211, 190)  # 8,018 and 40,090 rays: one batch, and three of which the last is ragged
 
 
@@ -47,10 +47,10 @@ def camera(size, row=0):
 
 
 @pytest.mark.parametrize("with_stats", [True, False])
-@pytest.mark.parametrize("D", [1, 8])
-def test_batches_equal_strips(fnr, D, with_stats):
+@pytest.mark.parametrize("D,n", [(1, N), (8, N), (4, N + 190)])
+def test_batches_equal_strips(fnr, D, n, with_stats):
     import torch
-    nets, p = networks(D), fnr.make_params(N, t_thr=0.3)
+    nets, p = networks(D), fnr.make_params(n, t_thr=0.3)
     ctx = fnr.fnr_context_create(0, 0)
     try:
         def render(cam):
@@ -65,7 +65,7 @@ def test_batches_equal_strips(fnr, D, with_stats):
             assert torch.equal(got, torch.cat(want))
         seen = torch.cat([s for _, s in strips]).reshape(-1, 4)
         if with_stats:
-            assert bool((seen[:, 0] < N).any()) and bool((seen[:, 3] == -1).all())
+            assert bool((seen[:, 0] < n).any()) and bool((seen[:, 3] == -1).all())
         else:
             assert bool((seen == -5).all())
         assert fnr.fnr_context_used_bytes(ctx) == 0
