@@ -367,10 +367,12 @@ FNR_API fnr_status fnr_render(fnr_context *ctx, const fnr_cache *cache, const fn
  * bmin_a <= p_a < bmax_a on every axis. F_pos reads the raw position (its
  * positional encoding as for the cache build); sigma = ReLU(output 0), u_i,
  * v_i, w_i = outputs 1..3D; F_dir reads the unit direction; beta = outputs
- * 0..D-1. One view per call; device temporaries are allocated per call and
- * charged to the budget. Stats: n_lookups = inside samples up to termination,
- * n_occupied = those with sigma > 0, dir_cell = -1. Errors: INVALID_ARG,
- * UNSUPPORTED, BUDGET, CUDA, DEVICE. */
+ * 0..D-1. One view per call, its rays in batches (8 Mi samples, or 16 Ki rays
+ * if that is more); the device temporaries are allocated per call, sized for
+ * one batch's samples, and charged to the budget. Stats: n_lookups = inside
+ * samples up to termination, n_occupied = those with sigma > 0, dir_cell = -1.
+ * A call that fails leaves rgba_dev and stats_dev as they were. Errors:
+ * INVALID_ARG, UNSUPPORTED, BUDGET, OOM, CUDA, DEVICE. */
 FNR_API fnr_status fnr_render_mlp(fnr_context *ctx, const fnr_mlp *pos_mlp, const fnr_mlp *dir_mlp, int32_t D,
                                   const float *bmin, const float *bmax, const fnr_camera *cam,
                                   const fnr_render_params *params, float *rgba_dev, fnr_ray_stats *stats_dev,

@@ -277,28 +277,26 @@ extern "C" fnr_status fnr_render_mlp(fnr_context *ctx, const fnr_mlp *pos_mlp, c
     FrameDesc F;
     fill_frame(&F, cam, rgba_dev, stats_dev, nullptr, 0);
     const long long n_rays = static_cast<long long>(cam->width) * cam->height;
-    // The budget is charged for temporaries of all samples at once; those of one batch are allocated, sized for
-    // every one of its samples.
-    const long long max_pts = n_rays * rc.N;
-    const uint64_t bytes = uint64_t(max_pts) * (3 + 1 + 3 * D) * 4 + uint64_t(n_rays) * (8 + 4 + 12 + 4 * D) + 8;
-    if (!budget_charge(ctx, bytes))
-        return fail(FNR_ERR_BUDGET, "the uncached render needs %llu bytes of temporaries",
-                    (unsigned long long)bytes);
     constexpr long long kBatchPoints = 1LL << 23, kBatchRays = 1LL << 14;
     const long long most = std::max<long long>(kBatchPoints / rc.N, kBatchRays);
     const long long n_batches = (n_rays + most - 1) / most, batch = (n_rays + n_batches - 1) / n_batches;
     const long long batch_pts = batch * rc.N;
     const bool staged = n_batches > 1;
+    // the batch's sample list and F_pos over it, the directions and F_dir over them, the rays' places in the list, the
+    // lists' lengths, the image
+    const size_t sizes[] = {size_t(batch_pts) * 12, size_t(batch_pts) * (1 + 3 * D) * 4, size_t(n_rays) * 12,
+                            size_t(n_rays) * D * 4, size_t(batch) * 8,                   size_t(n_batches) * 8,
+                            staged ? size_t(n_rays) * 16 : 0};
+    uint64_t bytes = 0;  // charged while the call runs
+    for (size_t v : sizes) bytes += v;
+    if (!budget_charge(ctx, bytes))
+        return fail(FNR_ERR_BUDGET, "the uncached render needs %llu bytes of temporaries", (unsigned long long)bytes);
     TempBuf points, pos_out, dirs, dir_out, offset, totals, image;
     PointsMlp pos, dir;
-    if ((e = points.alloc(ctx, size_t(batch_pts) * 12, s)) != cudaSuccess ||
-        (e = pos_out.alloc(ctx, size_t(batch_pts) * (1 + 3 * D) * 4, s)) != cudaSuccess ||
-        (e = dirs.alloc(ctx, size_t(n_rays) * 12, s)) != cudaSuccess ||
-        (e = dir_out.alloc(ctx, size_t(n_rays) * D * 4, s)) != cudaSuccess ||
-        (e = offset.alloc(ctx, size_t(batch) * 8, s)) != cudaSuccess ||
-        (e = totals.alloc(ctx, size_t(n_batches) * 8, s)) != cudaSuccess ||
-        (staged && (e = image.alloc(ctx, size_t(n_rays) * 16, s)) != cudaSuccess))
-        st = cuda_fail(e, "uncached render temporaries");
+    TempBuf *const bufs[] = {&points, &pos_out, &dirs, &dir_out, &offset, &totals, &image};
+    for (int i = 0; i < 7 && st == FNR_OK; ++i)
+        if (sizes[i] && (e = bufs[i]->alloc(ctx, sizes[i], s)) != cudaSuccess)
+            st = cuda_fail(e, "uncached render temporaries");
     if (st == FNR_OK && (e = cudaMemsetAsync(totals.p, 0, size_t(n_batches) * 8, s)) != cudaSuccess)
         st = cuda_fail(e, "memset");
     if (st == FNR_OK) st = pos.prepare(ctx, pos_mlp, 1 + 3 * D, true, s);

@@ -91,3 +91,25 @@ def test_failed_render_leaves_the_arrays(fnr, size):
         assert not bool((rgba.reshape(-1, 4) == 7.0).any()) and not bool((stats == -5).any())
     finally:
         fnr.fnr_context_destroy(ctx)
+
+
+def test_budget_is_charged_for_one_batch(fnr):
+    """The samples of the view would take 2.3 GB at once, a batch's 0.8: a budget between the two admits the view, one
+    below the batch does not, and either way nothing stays charged."""
+    import torch
+    nets, p, cam = networks(8), fnr.make_params(N), camera(SEVERAL)
+    images = []
+    for budget in (0, 1 << 30):
+        ctx = fnr.fnr_context_create(0, budget)
+        rgba, stats = arrays(*SEVERAL)
+        fnr.fnr_render_mlp(ctx, *nets, 8, cam, p, rgba, stats)
+        torch.cuda.synchronize()
+        images.append(rgba)
+        assert fnr.fnr_context_used_bytes(ctx) == 0
+        fnr.fnr_context_destroy(ctx)
+    assert torch.equal(*images)
+    ctx = fnr.fnr_context_create(0, 1 << 29)
+    with pytest.raises(fnr.FnrError) as ei:
+        fnr.fnr_render_mlp(ctx, *nets, 8, cam, p, rgba, stats)
+    assert ei.value.status == fnr.FNR_ERR_BUDGET and fnr.fnr_context_used_bytes(ctx) == 0
+    fnr.fnr_context_destroy(ctx)
