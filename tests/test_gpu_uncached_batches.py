@@ -113,3 +113,22 @@ def test_budget_is_charged_for_one_batch(fnr):
         fnr.fnr_render_mlp(ctx, *nets, 8, cam, p, rgba, stats)
     assert ei.value.status == fnr.FNR_ERR_BUDGET and fnr.fnr_context_used_bytes(ctx) == 0
     fnr.fnr_context_destroy(ctx)
+
+
+@pytest.mark.parametrize("size", [ONE, SEVERAL])
+def test_view_past_the_box(fnr, size):
+    """No ray reaches the box: F_pos has no samples at all, and the image is the background."""
+    import torch
+    nets, cam = networks(8), camera(size)
+    cam["c2w"] = np.array(cam["c2w"], np.float32)
+    cam["c2w"][3::4] += 100.0
+    p = fnr.make_params(N, bg=(0.25, 0.5, 0.75))
+    ctx = fnr.fnr_context_create(0, 0)
+    try:
+        rgba, stats = arrays(*size)
+        fnr.fnr_render_mlp(ctx, *nets, 8, cam, p, rgba, stats)
+        want = torch.tensor([0.25, 0.5, 0.75, 0.0], device="cuda")
+        assert bool((rgba.reshape(-1, 4) == want).all())
+        assert bool((stats.reshape(-1, 4) == torch.tensor([N, 0, 0, -1], device="cuda", dtype=torch.int32)).all())
+    finally:
+        fnr.fnr_context_destroy(ctx)
