@@ -54,12 +54,24 @@ constexpr int walk_group() {
     return PREC == FNR_PREC_FP8_E4M3 && FORM == kVoxJump ? 3 : 4;
 }
 
-// Minimum resident blocks per SM (registers against latency). FP32 with / without skipping at 6 / 7 / 8 blocks:
-// 640 / 613 / 581 and 994 / 932 / 886 us; FP16 without skipping (512 x 512, k = 256) 181 / 171 / 177; E4M3 with it
-// 720 / 719 / 704.
-template <int PREC, int FORM>
+// Minimum resident blocks per SM (registers against latency), by precision and record length. us at 5 / 6 / 7 / 8 blocks,
+// without and with skipping, 800 x 800, k = 350, and 512 x 512, k = 256:
+//   FP32 D = 8    629 568 535 516, 491 437 408 392;  204 188 180 177, 174 164 158 164
+//        D = 12   666 611 585 565, 568 547 533 545;  225 208 203 208, 227 226 232 246
+//        D = 16   738 679 635 620, 586 541 509 490;  261 245 239 246, 235 239 241 251
+//   FP16 D = 8    570 542 542 531, 498 446 414 391;  181 177 176 178, 179 170 163 167
+//        D = 12   679 631 601 604, 611 565 537 546;  213 202 196 201, 228 221 226 237
+//        D = 16   708 654 626 636, 563 506 473 454;  229 217 217 227, 212 207 209 218
+//   E4M3 D = 4    821 785 773 817, 562 530 506 503;  256 249 247 263, 225 222 217 229
+//        D = 8    677 655 674 691, 520 484 476 477;  218 215 227 237, 203 197 200 210
+//        D = 12   753 764 771 783, 668 676 690 709;  245 252 257 268, 268 290 315 323
+//        D = 16   850 889 888 894, 640 640 631 658;  278 304 319 340, 261 277 303 328
+// E4M3 records are decoded with their offsets and scales in registers: at 8 blocks (64 registers) its kernels spill up
+// to 550 bytes, so short ones run at 7 and long ones at 5. FP32 spills at most 44 bytes at 8 (D = 15: 220), FP16 24 at 7.
+template <int PREC, int D, int FORM>
 constexpr int walk_blocks() {
     if (FORM == kVoxCells || FORM == kVoxSkipCells) return 4;
+    if (PREC == FNR_PREC_FP8_E4M3) return D <= 8 ? 7 : 5;
     return PREC == FNR_PREC_FP16 ? 7 : 8;
 }
 
@@ -268,7 +280,7 @@ struct VoxelWalk {
 };
 
 template <int PREC, int D, int FORM>
-__global__ void __launch_bounds__(FNR_BLOCK, walk_blocks<PREC, FORM>())
+__global__ void __launch_bounds__(FNR_BLOCK, (walk_blocks<PREC, D, FORM>()))
     march_voxels_kernel(const __grid_constant__ MarchArgs A) {
     allow_next_grid();
     constexpr unsigned FULL = 0xffffffffu;
