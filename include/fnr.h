@@ -111,10 +111,16 @@ typedef struct fnr_cache fnr_cache;
 /* ------------------------------------------------------------------ context */
 /* Create a context on CUDA device `device`. hbm_budget_bytes caps the device
  * memory the context allocates for caches plus the outputs of admitted
- * serving requests (0 = no cap). Errors: INVALID_ARG (bad device), CUDA. */
+ * serving requests and the temporaries of fnr_render_mlp (0 = no cap). Outside
+ * the budget a context keeps a pool of at most 128 MiB between calls for the
+ * temporaries of builds and uncached renders; allocations that need its idle
+ * memory get it, and it goes with the context. Errors: INVALID_ARG (bad
+ * device), CUDA. */
 FNR_API fnr_status fnr_context_create(int32_t device, uint64_t hbm_budget_bytes, fnr_context **out);
 /* Stops the request loop (outstanding requests finish first), frees every
- * cache the context still owns and the context. NULL is a no-op. */
+ * cache the context still owns (which waits for the device, as fnr_cache_free
+ * does; without one the call waits for no other context's work) and the
+ * context. NULL is a no-op. */
 FNR_API fnr_status fnr_context_destroy(fnr_context *ctx);
 /* Bytes currently charged against the budget. */
 FNR_API uint64_t fnr_context_used_bytes(const fnr_context *ctx);

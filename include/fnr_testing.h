@@ -29,9 +29,10 @@ FNR_API fnr_status fnr_testing_fail_allocations(int32_t skip, int32_t count);
 /* Arms a fault for the next tensor-core cache-build launch (fnr_build_cache
  * with FNR_SRC_MLP, or fnr_render_mlp): every mbarrier wait in the kernel
  * gives up after wait_limit polls (instead of 2^22), and, if withhold_chunk is
- * >= 0, each CTA's weight producer withholds that chunk (counted from 0 in
- * the CTA's stream of 64-column weight chunks), so the MMA issuer's wait for
- * it runs out. The kernel then sets its error word, drains the copies and
+ * >= 0, each CTA's weight producer withholds that copy (counted from 0 in
+ * the CTA's stream of weights: blocks of up to 128 outputs x 128 inputs in the
+ * single-CTA form, 64-column chunks in the CTA-pair form), so the MMA issuer's
+ * wait for it runs out. The kernel then sets its error word, drains the copies and
  * tensor-core operations it has in flight, frees its tensor memory and
  * returns; the entry point returns FNR_ERR_DEVICE and releases the cache. The
  * hook disarms itself after one launch. Errors: INVALID_ARG for

@@ -30,8 +30,8 @@ namespace dev {
 // counts is how many warps are there to wait. Groups of 8 needed 72 registers and 288 queue entries a warp; with 5
 // (6 where the record is small) 56 registers hold a lane's state, 9 blocks fit instead of 7 and the queue leaves
 // 30 KB more to L1. 800 x 800, k = 512, N = 128, D = 8, groups of 8 at 7 (FP16: 8) blocks -> here, in us: FP32 95.8 ->
-// 87.7, with skipping 87.9 -> 78.4, bricks 100 -> 89; FP16 81.2 -> 78.1, 81.7 -> 76.6, bricks 103 -> 87; E4M3 94.8 ->
-// 91.7, 98.4 -> 90.6. 5 / 6 / 8 samples at 9 blocks, FP32: 87.7 / 90.0 / 93.4 (D = 8), 82.2 / 79.3 / 82.1 (6), 82.0 /
+// 87.7, with skipping 87.9 -> 76.1, bricks 100 -> 88; FP16 81.2 -> 76.7, 81.7 -> 73.6, bricks 103 -> 85; E4M3 94.8 ->
+// 86.7, 98.4 -> 86.7 (2 to 5 us of it by leaving the code for per-sample cells to CELLS). 5 / 6 / 8 samples at 9 blocks, FP32: 87.7 / 90.0 / 93.4 (D = 8), 82.2 / 79.3 / 82.1 (6), 82.0 /
 // 78.0 / 80.2 (4). E4M3 carries offsets and scales besides and spills at 9 blocks (110). Longer records need their
 // registers: FP32 at 7 / 8 / 9 blocks 101.6 / 94.8 / 99.4 (D = 12) and 118.8 / 115.6 / 118.0 (16). 800 x 800, k = 400,
 // groups of 6: E4M3 at 6 / 7 / 8 blocks 96.0 / 92.3 / 96.6 (D = 12), 101.5 / 97.2 / 101.0 (14), 110.2 / 100.2 / 116.2
@@ -203,12 +203,11 @@ __device__ __forceinline__ unsigned brick_occupied(const CacheView &c, int brick
 
 // floor(s * 2^32) of a binary32 s > 0: integer part and scaled fraction, both exact, each by one conversion to
 // 32 bits (to 64 bits they run on the FP64 pipe). s >= 2^31 gives 2^63 - 1: both conversions saturate, the second
-// because the first's result is rounded down on its way back (by a comparison and selects instead, the voxel walk of
-// an 800 x 800 view took 549 us, now 543). By shifts of the significand and
-// with a saturating sum (here the sum is unsigned: two terms below 2^63 cannot wrap, and the threshold ends the ray
-// after the first that reaches it) an 800 x 800 view took 96.2 / 82.2 / 96.4 us from FP32 / FP16 / E4M3 caches and
-// 109.1 from bricks, by conversions 95.9 / 81.3 / 94.9 and 100.2 (groups of 8 samples); the voxel walk of it 927 and
-// 875 us (groups of 8 cells).
+// because the first's result is rounded down on its way back (by a comparison and selects instead the voxel walk takes
+// 1% longer). By shifts of the significand and with a saturating sum (here the sum is unsigned: two terms below 2^63
+// cannot wrap, and the threshold ends the ray after the first that reaches it) an 800 x 800 view took 96.2 / 82.2 /
+// 96.4 us from FP32 / FP16 / E4M3 caches and 109.1 from bricks, by conversions 95.9 / 81.3 / 94.9 and 100.2 (groups of 8
+// samples); the voxel walk of it 927 and 875 us (groups of 8 cells).
 __device__ __forceinline__ unsigned long long fixed_depth(float s) {
     const int hi = __float2int_rz(s);
     const unsigned int lo = __float2uint_rz(__fmul_rn(__fsub_rn(s, __int2float_rz(hi)), 4294967296.0f));

@@ -10,14 +10,14 @@
 // them in walk order (weights, transmittance, exact fixed-point termination)
 // and only then loads the records of the cells it composited; a group with no
 // density in any lane of the warp ends at its density loads. What bounds it is
-// the issue of the walk's instructions (k = 352, skipping: 0.76 issued per
-// cycle and scheduler), so it is those that were cut: divisions through the
-// ray's reciprocals (divide_by), short groups, empty groups left early. 800 x
-// 800, k = 512, FP32: 1064 -> 875 us, with skipping 876 -> 543; FP16,
-// 512 x 512, k = 256: 230 -> 172, with skipping 265 -> 162; E4M3 with skipping
-// 1486 -> 675. In this mode the launcher passes
-// t_far in r.dt (the walk has no sample spacing) and r.s_thr is the threshold
-// on sum floor(fp32(sigma delta) 2^32).
+// the issue of the walk's instructions (k = 256, every cell / skipping: 0.76 /
+// 0.78 issued per cycle and scheduler), so it is those that were cut: divisions
+// through the ray's reciprocals (divide_by), short groups, empty groups left
+// early, no code for outputs that are not asked for. 800 x 800, k = 512, FP32:
+// 1064 -> 750 us, with skipping 876 -> 518; FP16, 512 x 512, k = 256: 230 -> 168,
+// with skipping 265 -> 156; E4M3 with skipping 1486 -> 646. In this mode the
+// launcher passes t_far in r.dt (the walk has no sample spacing) and r.s_thr is
+// the threshold on sum floor(fp32(sigma delta) 2^32).
 //
 // The kernel is instantiated four times per (precision, D), one form per
 // translation unit: the plain walk (march_voxels.cu), the walk that skips the

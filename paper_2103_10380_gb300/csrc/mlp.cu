@@ -174,7 +174,7 @@ __device__ __forceinline__ uint32_t bias_relu_bf16(uint32_t a, uint32_t b, float
 
 // 32 accumulator columns from output n0 on -> 16 columns of A: ReLU(acc + bias) as bf16, outputs past N as 0.
 // bias: shared-memory address of output 0's. (The loads are volatile so that they stay beside their use: hoisted,
-// they push the warp's 80 registers over into local memory.)
+// they push the warp's 80 registers over into local memory by far more than the 20 bytes that ptxas spills now.)
 __device__ __forceinline__ void relu_columns(const uint32_t (&r)[32], uint32_t bias, int n0, int N, uint32_t (&pk)[16]) {
 #pragma unroll
     for (int u = 0; u < 32; u += 16) {
