@@ -210,7 +210,8 @@ FNR_API uint64_t fnr_cache_bytes(const fnr_cache_desc *desc);
  * and the occupancy bits. For FNR_LAYOUT_BRICKS it is the bound with every
  * brick stored; a built cache reports its own footprint (fnr_cache_get_layout).
  * A BRICKS build passes through a dense cache, which is charged to the budget
- * while it exists. */
+ * while it exists (from device arrays through one without records, charged all
+ * the same). */
 FNR_API uint64_t fnr_cache_footprint(const fnr_cache_desc *desc);
 
 /* Build a cache on `stream`. Returns when the cache is complete (the call
